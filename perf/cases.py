@@ -49,8 +49,8 @@ def listed():
         _case("solve_256_thirds", "solve", 3, 4, 32, 256, 6, 3, 4, K=2, J=4, precision=0),
         # 8 shots with a 6x6 filter: the largest Gram (C = 288) of the batched workload, a short schedule too
         _case("solve_192_8shots", "solve", 2, 8, 16, 192, 6, 2, 2, K=3, J=5, precision=0),
-        # one gradient of the learned warm start's network on two slice groups of 12 slice-shots
-        _case("cnn_gradients_256", "cnn", 3, 4, 0, 256, 0, 0, 2, width=64, layers=6),
+        # the learned warm start's network applied to the k-space of two slice groups before their solve
+        _case("learned_start_256", "start", 3, 4, 2, 256, 6, 3, 2, width=64, layers=6),
     ]
 
 
@@ -62,7 +62,7 @@ def draw(rng):
     """One more case: any of the operations, geometry over the workloads' whole range (matrices 48 to 256 with
     factors of 3 among them, 1 to 3 slices, 1 to 8 shots, 2 to 32 coils), batches up to the cost of the largest."""
     while True:
-        op = rng.choice(["forward", "adjoint", "gram", "penalty", "sense", "solve", "solve", "cnn"])
+        op = rng.choice(["forward", "adjoint", "gram", "penalty", "sense", "solve", "solve", "start"])
         N = rng.choice([48, 64, 72, 96, 108, 128, 144, 192, 256])
         Ns = rng.choice([1, 2, 3, 4, 6, 8])
         if N % Ns or (N // Ns) % 2 or N // Ns < 8:
@@ -72,15 +72,12 @@ def draw(rng):
         r = rng.randint(2, {1: 9, 2: 8, 3: 6, 4: 6, 6: 6, 8: 6}[Ns])
         div = rng.choice([L, L, 2, 3, 4])
         pixels = L * Ns * N * N
-        if op == "cnn":
-            H = rng.choice([48, 64, 100, 128])
-            n = _log(rng, 1, 4)
-            B, width = L * Ns, rng.choice([16, 24, 48, 64])
-            return _case(None, "cnn", L, Ns, 0, H, 0, 0, n, width=width, layers=rng.randint(2, 6)) if B <= 24 else _case(
-                None, "cnn", 3, 4, 0, H, 0, 0, n, width=width, layers=3)
         D = _log(rng, 1, max(1, min(26, int(26 * 2 * 4 * 128 * 128 / pixels))))
         more = {}
-        if op == "sense":
+        if op == "start":
+            D, Nc = min(D, max(1, 2 * 256 * 256 // (N * N))), 2
+            more = {"width": rng.choice([16, 24, 40, 48, 64]), "layers": rng.randint(2, 6)}
+        elif op == "sense":
             more = {"J": rng.randint(3, 30), "phase": rng.random() < 0.5}
         elif op == "solve":
             C = Ns * r * r
@@ -168,19 +165,9 @@ def _inputs(c, seed):
     """The tensors a call takes, by name, rounded to its types: a pure function of the case and the seed."""
     op, D, L, Ns, Nc, N = c["op"], c["D"], c["L"], c["Ns"], c["Nc"], c["N"]
     g = _gen(seed + 1000003)
-    if op == "cnn":
-        B, w, n = L * Ns, c["width"], c["layers"]
-        img, _ = _images(c, seed)
-        t = img.reshape(D, B, N, N)
-        t = t / torch.sqrt((t.abs() ** 2).mean())
-        params = []
-        for k in range(n):
-            ci, co = (B if k == 0 else w), (B if k + 1 == n else w)
-            params += [(_crandn(g, co * ci * 9) / math.sqrt(9 * ci)), 0.01 * _crandn(g, co)]
-        return {"a": _c64(t + 0.3 * _crandn(g, *t.shape)), "t": _c64(t), "params": _c64(torch.cat(params))}
     img, ph = _images(c, seed)
     out = {"sens": _c64(_coils(L, Nc, N))}
-    if op in ("gram", "penalty", "forward"):
+    if op in ("gram", "penalty", "forward", "start"):
         x = _fft2c(img)
         out["x"] = _c64(_lead(c, x / torch.sqrt((x.abs() ** 2).mean())))
         if op == "penalty":
@@ -188,6 +175,12 @@ def _inputs(c, seed):
             A = _crandn(g, D, L, C, max(1, C // 2)) / math.sqrt(C)
             W = 0.1 * torch.eye(C, device=DEV, dtype=torch.complex128) + A @ A.mH  # a weight: Hermitian, positive
             out["W"] = _lead(c, 0.5 * (W + W.mH)).contiguous()
+        if op == "start":
+            params, w, n = [], c["width"], c["layers"]
+            for k in range(n):
+                ci, co = (L * Ns if k == 0 else w), (L * Ns if k + 1 == n else w)
+                params += [(_crandn(g, co * ci * 9) / math.sqrt(9 * ci)), 0.01 * _crandn(g, co)]
+            out["params"] = _c64(torch.cat(params))
         return out
     S = out["sens"].to(torch.complex128)
     y = torch.stack([_forward(_fft2c(v), S, c["div"]) for v in img])
@@ -205,15 +198,14 @@ def _inputs(c, seed):
 def prepare(case, seed):
     c, v = case, _inputs(case, seed)
     s = dict(v, case=c)
-    if c["op"] == "cnn":
-        s["net"] = smsm.CNN(c["L"] * c["Ns"], c["N"], c["N"], width=c["width"], layers=c["layers"], max_batch=c["D"])
-        s["net"].set_params(v["params"])
-        return s
     s["plan"] = smsm.Plan(c["L"], c["Ns"], c["Nc"], c["N"], c["r"], caipi_div=c["div"], batch=c["D"],
                           precision=c.get("precision", 0))
     s["plan"].set_sens(v["sens"])
     if c["op"] == "solve":
         s["params"] = smsm.default_params(lam=LAM, outer_iters=c["K"], cg_iters=c["J"])
+    if c["op"] == "start":
+        s["net"] = smsm.CNN(c["L"] * c["Ns"], c["N"], c["N"], width=c["width"], layers=c["layers"], max_batch=c["D"])
+        s["net"].set_params(v["params"])
     return s
 
 
@@ -232,8 +224,7 @@ def run(s):
     if op == "solve":
         x = s["plan"].reconstruct(s["y"], params=s["params"], report=False)[0]
         return list(x) if s["case"]["D"] > 1 else x  # one output per direction
-    loss, grad = s["net"].gradients(s["a"], s["t"])
-    return {"loss": loss, "grad": grad}
+    return smsm.learned_start(s["plan"], s["net"], s["x"])
 
 
 # --- what a pass cannot do without ---------------------------------------------------------------
@@ -244,12 +235,9 @@ def work(case):
     D, L, Ns, Nc, N, r = c["D"], c["L"], c["Ns"], c["Nc"], c["N"], c["r"]
     B, NN = L * Ns, N * N
     fft = 10 * NN * math.log2(N)  # one N x N transform
-    if c["op"] == "cnn":
-        w, n = c["width"], c["layers"]
-        mac = 9 * (B * w * 2 + w * w * (n - 2)) if n > 1 else 9 * B * B
-        first = 9 * B * (w if n > 1 else B)
-        # forward, weight gradient, data gradient (all layers but the first)
-        return {"bytes": 8 * (2 * D * B * NN + 2 * mac), "flops": 8 * D * NN * (3 * mac - first)}
+    if c["op"] == "start":
+        mac = 9 * (2 * B * c["width"] + c["width"] ** 2 * (c["layers"] - 2))
+        return {"bytes": 8 * (2 * D * B * NN + mac), "flops": D * (8 * NN * mac + 2 * B * fft)}
     x, y, sens, C, R2 = 8 * D * B * NN, 8 * D * Nc * NN, 8 * L * Nc * NN, Ns * r * r, 2 * r - 1
     P = (N - r + 1) ** 2
     # per coil, slice and shot: the coil products and, along y, the N/Ns-point transform of the kept lines; per coil
@@ -367,35 +355,31 @@ def _solve(y, S, c):
     return x
 
 
-def _cnn_exact(c, v):
+def _start(x, params, c):
+    """[L][Ns][N][N] k-space -> F(a + f(a)), a = F^-1 x; products take the weights rounded to BF16"""
     B, w, n = c["L"] * c["Ns"], c["width"], c["layers"]
-    p = torch.view_as_real(v["params"]).to(torch.bfloat16).double().requires_grad_(True)
-    a, t = (torch.cat([z.real, z.imag], 1).double() for z in (v["a"], v["t"]))
-    h, at = a, 0
+    p = torch.view_as_real(params).to(torch.bfloat16).double()
+    img = _ifft2c(x).reshape(1, B, c["N"], c["N"])
+    h, at = torch.cat([img.real, img.imag], 1), 0
     for k in range(n):
         ci, co = (B if k == 0 else w), (B if k + 1 == n else w)
         re, im = (p[at:at + co * ci * 9, j].reshape(co, ci, 3, 3) for j in (0, 1))
         at += co * ci * 9
+        W = torch.cat([torch.cat([re, -im], 1), torch.cat([im, re], 1)], 0)
         bias = torch.cat([p[at:at + co, 0], p[at:at + co, 1]])
         at += co
-        W = torch.cat([torch.cat([re, -im], 1), torch.cat([im, re], 1)], 0)
-        h = torch.nn.functional.conv2d(torch.relu(h) if k else h, W, bias, padding=1)
-    e, q = ((z ** 2).sum((1, 2, 3)) for z in (a + h - t, t))
-    loss = (e / q).mean()
-    (grad,) = torch.autograd.grad(loss, p)
-    return {"loss": float(loss), "grad": torch.view_as_complex(grad.contiguous())}
+        with torch.backends.cudnn.flags(enabled=False):  # native double convolution
+            h = torch.nn.functional.conv2d(torch.relu(h) if k else h, W, bias, padding=1)
+    return _fft2c((img + torch.complex(h[:, :B], h[:, B:])).reshape(x.shape))
 
 
 def exact(case, seed):
     c = case
     v = _inputs(c, seed)
-    if c["op"] == "cnn":
-        with torch.backends.cudnn.flags(enabled=False):  # native double convolutions
-            return _cnn_exact(c, v)
     up = {k: t.to(torch.complex128) for k, t in v.items()}
     S, D = up["sens"], c["D"]
     if D == 1:
-        up = {k: (t if k == "sens" else t[None]) for k, t in up.items()}
+        up = {k: (t if k in ("sens", "params") else t[None]) for k, t in up.items()}
     ph = up.get("phase")
     got = []
     for d in range(D):
@@ -407,6 +391,8 @@ def exact(case, seed):
             got.append(torch.stack([h.mH @ h for h in (_hankel(x, c["r"]) for x in up["x"][d])]))
         elif c["op"] == "penalty":
             got.append(_penalty(up["x"][d], up["W"][d], c["r"]))
+        elif c["op"] == "start":
+            got.append(_start(up["x"][d], v["params"], c))
         elif c["op"] == "solve" and d >= 3:
             got.append(None)  # three directions of a series say it
         elif c["op"] == "sense":

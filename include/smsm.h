@@ -100,13 +100,19 @@ typedef enum { SMSM_BOUNDARY_VALID = 0, SMSM_BOUNDARY_PERIODIC = 1 } smsm_bounda
  *                    per-class coil correlations (which need N % caipi_div == 0);
  *   CLUSTER_EIG: the eigen step by one-sided block Jacobi on a cluster of eight
  *                CTAs per Gram (C = shots*filter^2 >= 65) even where the two-CTA
- *                two-sided solver fits.  C > 168 always takes the cluster solver
+ *                two-sided solver fits or no eigen-decomposition is needed.  An
+ *                eigen-decomposition at C > 168 always takes the cluster solver
  *                (G of up to 320 x 320 does not fit one CTA's shared memory). */
 #define SMSM_FLAG_GENERIC_KERNELS 1
 #define SMSM_FLAG_PER_COIL_NORMAL 2
 #define SMSM_FLAG_CLUSTER_EIG 4
 
 /*
+ * The IRLS weights W_l = (G_l + eps I)^(-1/2) are formed without an eigen-decomposition
+ * unless the call asks for one (NULLSPACE mode, eig_cold, eig_tol > 0, max_sweeps below
+ * 30, SMSM_FLAG_CLUSTER_EIG, SMSM_FLAG_GENERIC_KERNELS), eps0_rel * eps_min_rel is below
+ * 1e-5, or a Gram's scale passes 2^20 eps; then the Jacobi eigensolvers make them.
+ *
  * Solver parameters.  The paper minimises Eq. 10 with an augmented-Lagrangian
  * scheme whose listing is in another paper; this library minimises the same
  * cost by IRLS: at outer iteration k the nuclear norm is majorised with
@@ -154,9 +160,11 @@ typedef struct {
 typedef enum {
   SMSM_STAGE_ADJOINT = 0,    /* b = A^H y (row FFT, column stage, row FFT) */
   SMSM_STAGE_GRAM = 1,       /* Hankel Gram partials + reduction */
-  SMSM_STAGE_EIG = 2,        /* Jacobi sweeps on G */
-  SMSM_STAGE_VAPPLY = 3,     /* Newton-Schulz re-orthonormalisation of V */
-  SMSM_STAGE_WEIGHTS = 4,    /* eps schedule + W */
+  SMSM_STAGE_EIG = 2,        /* eps schedule and W without an eigen-decomposition, or the Jacobi
+                                sweeps on G */
+  SMSM_STAGE_VAPPLY = 3,     /* Newton-Schulz re-orthonormalisation of V (and the eigensolver for
+                                matrices left to it) */
+  SMSM_STAGE_WEIGHTS = 4,    /* eps schedule + W from the eigenvectors */
   SMSM_STAGE_FILTERS = 5,    /* filters from W + image-domain multipliers */
   SMSM_STAGE_ROWFFT_INV = 6, /* x-direction inverse FFT of the CG vector */
   SMSM_STAGE_COLUMN = 7,     /* fused column stage of (A^H A + lambda P_W) */
@@ -175,7 +183,8 @@ typedef struct {
   double eps[SMSM_MAX_OUTER];           /* eps_k (IRLS) */
   double rr_start[SMSM_MAX_OUTER];      /* ||r||^2 at the start of outer k's CG */
   double rr_end[SMSM_MAX_OUTER];        /* ||r||^2 after its cg_iters steps */
-  int sweeps[SMSM_MAX_OUTER];           /* Jacobi sweeps used (max over slices) */
+  int sweeps[SMSM_MAX_OUTER];           /* Jacobi sweeps used (max over slices); 0 where the weights
+                                           were formed without an eigen-decomposition */
   float elapsed_ms;                     /* device time of the solve (CUDA events) */
   int graph_kernels;                    /* kernel launches in one solve (nodes of its graph) */
   float stage_ms[16];                   /* device time per smsm_stage (timed stages only; with

@@ -89,6 +89,18 @@ struct DevReport {
   int sweeps[SMSM_MAX_OUTER];
 };
 
+// The weights' quadrature (invsqrt.cu): W = wscale sum_j a_j ((G inv_c) + (shift + b_j) I)^(-1)
+#define IS_MAXN 16  // terms at most
+#define IS_MAXQ 20  // largest condition number c/eps taken: 2^20
+struct IsRow {  // nodes for [2^-q, 1]
+  int n;
+  float a[IS_MAXN], b[IS_MAXN];
+};
+struct IsParam {  // one Hankel matrix's
+  float inv_c, shift, wscale;
+  int q, n;  // row of the table, terms (0: left to the eigensolver)
+};
+
 // Maximum sizes of this build.
 #define SMSM_MAX_C 320
 #define SMSM_MAX_N 512
@@ -136,6 +148,12 @@ struct smsm_plan_s {
   int* sweeps;       // [L]
   float2 *V, *Wf;    // [LD][C][C]
   float2 *Gw, *Gw2;  // [LD][C][C] warm-start congruence V^H G V (and its half product)
+  float2* is_rows;   // [LD][C] row sums of |G| and |G|^2
+  float* is_lmax;    // [LD] largest eigenvalue of the first Gram
+  IsParam* is_prm;   // [LD]
+  IsRow* is_tab;     // [IS_MAXQ + 1]
+  float2* is_part;   // [matrices][IS_MAXN][blocks][16][16] terms of the sum (invsqrt_part_count)
+  int* is_flag;      // [LD] 1: this matrix's weight comes from the eigensolver
   float2* wper;      // [L][Ns][Ns][R2*R2]
   float2* wcls;      // [LD][R2*R2 classes][Ns (i')][R2*R2 taps][Ns (i)] border correction taps
   float2* multT;     // [L][Ns(Ns+1)/2][N(x)][N(y)]: upper triangle of the Hermitian shot coupling
@@ -289,7 +307,15 @@ bool eig_pair_supported(int Cp);
 bool eig_cluster_supported(int C);
 smsm_status eig_cluster_init_attrs(int C);
 smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const float2* T, int max_sweeps, float tol,
-                               float floor_rel, cudaStream_t s);
+                               float floor_rel, const int* only, cudaStream_t s);
+// invsqrt.cu
+const std::vector<IsRow>& invsqrt_table();
+size_t invsqrt_part_count(const smsm_plan_s* P);
+size_t invsqrt_part_offset(const smsm_plan_s* P, int d0, int lane);
+smsm_status invsqrt_init_attrs(const smsm_plan_s* P);
+bool invsqrt_applies(const smsm_plan_s* P, const smsm_params* prm);
+smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, const smsm_params* prm, cudaStream_t s,
+                           Timer* T);
 smsm_status operators_init_attrs();
 size_t smsm_col_smem_bytes(const smsm_plan_s* P);
 int band_blocks(const smsm_plan_s* P);

@@ -94,7 +94,8 @@ __host__ __device__ inline size_t jac_smem_bytes(int Cp) { return jac_region_a(C
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(1024)
     k_jacobi(const double2* __restrict__ G, const float2* __restrict__ Gw, float* __restrict__ eig,
              float2* __restrict__ V, int warmv, int* __restrict__ sweeps_out, int C, int Cp, int max_sweeps, float tol,
-             float floor_rel, SolverState* st, int L, int* __restrict__ errflag) {
+             float floor_rel, SolverState* st, int L, int* __restrict__ errflag, const int* __restrict__ only) {
+  if (only && !only[blockIdx.x >> 1]) return;  // both CTAs of the cluster alike
   extern __shared__ __align__(16) unsigned char jsm[];
   __shared__ __align__(8) uint64_t full_b[2], empty_b[2];
   __shared__ int hdr[2];
@@ -389,7 +390,12 @@ template <int OP>
 __global__ void __launch_bounds__(256) k_cgemm(const double2* __restrict__ G, const float2* __restrict__ X,
                                                const float2* __restrict__ Y, float2* __restrict__ out, int C,
                                                const float* __restrict__ eig, const SolverState* __restrict__ st,
-                                               int Cp, int mode, int rank, int L) {
+                                               int Cp, int mode, int rank, int L, const int* __restrict__ only, int* rep_sweeps,
+                                               const int* __restrict__ sweeps) {
+  if (only && !only[blockIdx.z]) return;
+  // the report follows direction 0: its slices are matrices 0 .. L - 1
+  if (OP == SG_W && rep_sweeps && blockIdx.z < L && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+    atomicMax(rep_sweeps, sweeps[blockIdx.z]);
   __shared__ float2 As[SG_T][SG_K + 1];
   __shared__ float2 Bs[SG_K][SG_T + 1];
   __shared__ float f[OP == SG_W ? SMSM_MAX_C : 1];
@@ -486,11 +492,12 @@ __global__ void __launch_bounds__(256) k_cgemm(const double2* __restrict__ G, co
 
 template <int OP>
 static smsm_status launch_cgemm(const smsm_plan_s* P, const double2* G, const float2* X, const float2* Y,
-                                float2* out, const smsm_params* prm, cudaStream_t s) {
+                                float2* out, const smsm_params* prm, cudaStream_t s,
+                                const int* only = nullptr, int* rep_sweeps = nullptr) {
   const int C = P->C;
   const dim3 grid((C + SG_T - 1) / SG_T, (C + SG_T - 1) / SG_T, P->LD);
   k_cgemm<OP><<<grid, 256, 0, s>>>(G, X, Y, out, C, P->eig, P->st, P->Cp, prm ? prm->mode : 0, prm ? prm->rank : 0,
-                                   P->L);
+                                   P->L, only, rep_sweeps, P->sweeps);
   SMSM_LAUNCH_CHECK("k_cgemm");
   return SMSM_OK;
 }
@@ -563,13 +570,34 @@ smsm_status launch_eig_weights(const smsm_plan_s* P, const double2* G, int outer
   if (msw > SMSM_MAX_SWEEPS) msw = SMSM_MAX_SWEEPS;
   // warm start from the previous outer iteration's eigenvectors (same solve)
   const int warm = (outer > 0 && !prm->eig_cold) ? 1 : 0;
-  if (T) T->begin(SMSM_STAGE_EIG);
   smsm_status sg;
+  if (invsqrt_applies(P, prm)) {
+    if ((sg = launch_invsqrt(P, G, outer, prm, s, T))) return sg;
+    // the matrices it left: eigenvectors from scratch, V re-orthonormalised, W (the launches
+    // return at once for every other matrix)
+    const int* only = P->is_flag;
+    if (T) T->begin(SMSM_STAGE_VAPPLY);
+    if (P->eig_cluster) {
+      if ((sg = launch_eig_cluster(P, G, nullptr, msw, 2e-6f, 1e-12f, only, s))) return sg;
+    } else {
+      k_jacobi<<<2 * P->LD, 1024, jac_smem_bytes(Cp), s>>>(G, nullptr, P->eig, P->V, 0, P->sweeps, C, Cp, msw, 1e-6f,
+                                                            1e-12f, P->st, P->L, P->devflag, only);
+      SMSM_LAUNCH_CHECK("k_jacobi");
+    }
+    if ((sg = launch_cgemm<SG_VHV>(P, nullptr, P->V, nullptr, P->Gw, prm, s, only))) return sg;
+    if ((sg = launch_cgemm<SG_NS>(P, nullptr, P->V, P->Gw, P->Gw2, prm, s, only))) return sg;
+    if ((sg = launch_cgemm<SG_W>(P, nullptr, P->Gw2, nullptr, P->Wf, prm, s, only,
+                                  outer < SMSM_MAX_OUTER ? P->rep->sweeps + outer : nullptr)))
+      return sg;
+    if (T) T->end(SMSM_STAGE_VAPPLY);
+    return SMSM_OK;
+  }
+  if (T) T->begin(SMSM_STAGE_EIG);
   if (P->eig_cluster) {
     // one-sided Jacobi on A = G V_prev (the congruence's first product) or on G itself
     if (warm && (sg = launch_cgemm<SG_GV>(P, G, P->V, nullptr, P->Gw, prm, s))) return sg;
     const float tol = prm->eig_tol > 0.f ? prm->eig_tol : 2e-6f;
-    smsm_status st = launch_eig_cluster(P, G, warm ? P->Gw : nullptr, msw, tol, 1e-12f, s);
+    smsm_status st = launch_eig_cluster(P, G, warm ? P->Gw : nullptr, msw, tol, 1e-12f, nullptr, s);
     if (st) return st;
   } else {
   if (warm) {
@@ -584,7 +612,7 @@ smsm_status launch_eig_weights(const smsm_plan_s* P, const double2* G, int outer
   // two CTAs per matrix: the Jacobi rounds on G and, beside them, V times every rotation
   k_jacobi<<<2 * P->LD, 1024, jac_smem_bytes(Cp), s>>>(G, warm ? P->Gw2 : nullptr, P->eig, P->V, warm, P->sweeps, C,
                                                         Cp, msw, prm->eig_tol > 0.f ? prm->eig_tol : 1e-6f,
-                                                        (float)frel, P->st, P->L, P->devflag);
+                                                        (float)frel, P->st, P->L, P->devflag, nullptr);
   SMSM_LAUNCH_CHECK("k_jacobi");
   }
   if (T) T->end(SMSM_STAGE_EIG);

@@ -142,7 +142,8 @@ template <int KR>
 __global__ void __cluster_dims__(OSJ_R, 1, 1) __launch_bounds__(640, 1)
     k_jacobi_os(const double2* __restrict__ G, const float2* __restrict__ T, float* __restrict__ eig,
                 float2* __restrict__ V, int* __restrict__ sweeps_out, int C, int Cp, int max_sweeps, float tol,
-                float floor_rel, SolverState* st, int L) {
+                float floor_rel, SolverState* st, int L, const int* __restrict__ only) {
+  if (only && !only[blockIdx.x / OSJ_R]) return;  // every CTA of the cluster alike
   extern __shared__ __align__(16) float2 osm[];
   __shared__ int vote[OSJ_R];
   __shared__ float dmax_s;
@@ -266,7 +267,7 @@ __global__ void __cluster_dims__(OSJ_R, 1, 1) __launch_bounds__(640, 1)
 }
 
 typedef void (*OsjFn)(const double2*, const float2*, float*, float2*, int*, int, int, int, float, float,
-                      SolverState*, int);
+                      SolverState*, int, const int*);
 
 static OsjFn osj_fn(int C) {
   switch (osj_kr(C)) {
@@ -302,11 +303,11 @@ smsm_status eig_cluster_init_attrs(int C) {
 }
 
 smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const float2* T, int max_sweeps, float tol,
-                               float floor_rel, cudaStream_t s) {
+                               float floor_rel, const int* only, cudaStream_t s) {
   OsjFn fn = osj_fn(P->C);
   if (!fn) return SMSM_ERR_ARG;
   fn<<<OSJ_R * P->LD, 32 * osj_w(P->C), osj_smem(P->C), s>>>(G, T, P->eig, P->V, P->sweeps, P->C, P->Cp, max_sweeps,
-                                                             tol, floor_rel, P->st, P->L);
+                                                             tol, floor_rel, P->st, P->L, only);
   SMSM_LAUNCH_CHECK("k_jacobi_os");
   return SMSM_OK;
 }

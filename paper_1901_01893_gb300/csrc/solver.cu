@@ -300,6 +300,11 @@ static smsm_plan_s lane_view(const smsm_plan_s* P, int d0, int nd, int lane) {
   v.Wf += cc;
   v.Gw += cc;
   v.Gw2 += cc;
+  v.is_rows += dd * L * C;
+  v.is_lmax += dd * L;
+  v.is_prm += dd * L;
+  v.is_flag += dd * L;
+  v.is_part += invsqrt_part_offset(P, d0, lane);
   v.Gpart += cc * P->gram_nkx;
   v.eig += dd * L * Cp;
   v.sweeps += dd * L;

@@ -97,7 +97,7 @@ static void free_plan(smsm_plan_s* P) {
                   P->G64,  P->Gpart, P->eig,    P->sweeps, P->V,   P->Wf,   P->wper, P->Gw, P->Gw2,
                   P->wcls, P->multT, P->part_pq_col, P->part_pq_band, P->part_rr, P->st, P->rep,
                   P->Rpart, P->devflag, P->acorr, P->ash, P->is_rows, P->is_lmax, P->is_prm,
-                  P->is_flag, P->is_tab, P->is_part};
+                  P->is_flag, P->is_tab, P->scratch};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   solver_forget_plan(P);
@@ -243,7 +243,7 @@ extern "C" smsm_status smsm_plan(smsm_plan_t* out, int mb, int shots, int coils,
   A(is_prm, LD);
   A(is_flag, LD);
   A(is_tab, IS_MAXQ + 1);
-  A(is_part, invsqrt_part_count(P));
+  A(scratch, scratch_count(P));
   A(wper, LD * shots * shots * R2 * R2);
   A(wcls, LD * R2 * R2 * shots * shots * R2 * R2);
   A(multT, LD * mult_planes(shots) * NN);
@@ -335,6 +335,7 @@ extern "C" smsm_status smsm_plan(smsm_plan_t* out, int mb, int shots, int coils,
   }
   if (!st) st = upload(P->is_tab, invsqrt_table());
   if (!st) st = invsqrt_init_attrs(P);
+  if (!st) st = gram_lag_init_attrs(P);
   if (!st) st = operators_init_attrs();
   if (!st) st = colfast_init_attrs();
   if (!st) st = alias_init_attrs();

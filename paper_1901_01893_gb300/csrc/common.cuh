@@ -57,6 +57,12 @@ __device__ __forceinline__ void cp_async8(void* dst_smem, const void* src) {
                "l"(src)
                : "memory");
 }
+// the same, writing zero instead when !valid (src stays a readable address)
+__device__ __forceinline__ void cp_async8_zero(void* dst_smem, const void* src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)),
+               "l"(src), "r"(valid ? 8 : 0)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
 }
@@ -152,7 +158,7 @@ struct smsm_plan_s {
   float* is_lmax;    // [LD] largest eigenvalue of the first Gram
   IsParam* is_prm;   // [LD]
   IsRow* is_tab;     // [IS_MAXQ + 1]
-  float2* is_part;   // [matrices][IS_MAXN][blocks][16][16] terms of the sum (invsqrt_part_count)
+  float2* scratch;   // per matrix: the Gram's lagged sums, then the weights' terms (scratch_count)
   int* is_flag;      // [LD] 1: this matrix's weight comes from the eigensolver
   float2* wper;      // [L][Ns][Ns][R2*R2]
   float2* wcls;      // [LD][R2*R2 classes][Ns (i')][R2*R2 taps][Ns (i)] border correction taps
@@ -292,6 +298,11 @@ int gram_tc_nG(const smsm_plan_s* P);
 int gram_tc_nG_candidates(const smsm_plan_s* P, int* out, int maxn);
 smsm_status gram_tc_init_attrs();
 smsm_status launch_gram_tc(const smsm_plan_s* P, const float2* x, double2* G, cudaStream_t s);
+// gram_lag.cu
+int gram_lag_supported(const smsm_plan_s* P);
+size_t gram_lag_per(const smsm_plan_s* P);
+smsm_status gram_lag_init_attrs(const smsm_plan_s* P);
+smsm_status launch_gram_lag(const smsm_plan_s* P, const float2* x, double2* G, cudaStream_t s);
 smsm_status launch_filters(const smsm_plan_s* P, const float2* W, cudaStream_t s);
 smsm_status launch_band(const smsm_plan_s* P, const float2* x, float2* out, float scale, double* dot_part,
                         cudaStream_t s);
@@ -310,8 +321,7 @@ smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const flo
                                float floor_rel, const int* only, cudaStream_t s);
 // invsqrt.cu
 const std::vector<IsRow>& invsqrt_table();
-size_t invsqrt_part_count(const smsm_plan_s* P);
-size_t invsqrt_part_offset(const smsm_plan_s* P, int d0, int lane);
+size_t invsqrt_per(const smsm_plan_s* P);
 smsm_status invsqrt_init_attrs(const smsm_plan_s* P);
 bool invsqrt_applies(const smsm_plan_s* P, const smsm_params* prm);
 smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, const smsm_params* prm, cudaStream_t s,
@@ -324,6 +334,8 @@ smsm_status band_init_attrs(const smsm_plan_s* P);
 smsm_status cnn_shape(const smsm_cnn_s* c, int* B, int* H, int* W, int* maxn);
 // solver.cu
 int vec_blocks(const smsm_plan_s* P);
+int scratch_cap(const smsm_plan_s* P);
+size_t scratch_count(const smsm_plan_s* P);
 smsm_status solver_reconstruct(smsm_plan_s* P, const void* y, void* x, const smsm_params* prm,
                                smsm_report* report, cudaStream_t s);
 smsm_status solver_autotune(smsm_plan_s* P, const void* y, const smsm_params* prm, smsm_tune_report* out,

@@ -547,26 +547,9 @@ bool invsqrt_applies(const smsm_plan_s* P, const smsm_params* prm) {
 
 static int rat_nb(int C) { return (C + RB - 1) / RB; }
 
-static size_t rat_per(int C) {  // one matrix's terms
-  const size_t nb = rat_nb(C);
+size_t invsqrt_per(const smsm_plan_s* P) {  // complex values of one matrix's terms
+  const size_t nb = rat_nb(P->C);
   return (size_t)IS_MAXN * (nb * (nb + 1) / 2) * RB * RB;
-}
-
-// matrices whose terms are formed in one launch at most: 96 MB of terms
-static int rat_cap(int C) {
-  const size_t n = (size_t)96 * 1024 * 1024 / (rat_per(C) * sizeof(float2));
-  return n < 1 ? 1 : (int)n;
-}
-
-// The terms' buffer: room for every matrix of the plan, or, when that is more than a launch takes, one
-// launch's room per lane.  Lane `lane` (directions from d0 on) owns what begins at the offset.
-size_t invsqrt_part_count(const smsm_plan_s* P) {
-  const size_t cap = rat_cap(P->C);
-  return rat_per(P->C) * ((size_t)P->LD <= cap ? (size_t)P->LD : cap * SMSM_MAX_LANES);
-}
-size_t invsqrt_part_offset(const smsm_plan_s* P, int d0, int lane) {
-  const size_t cap = rat_cap(P->C);
-  return rat_per(P->C) * ((size_t)P->LD <= cap ? (size_t)d0 * P->L : cap * lane);
 }
 
 typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int, int, int);
@@ -632,7 +615,7 @@ smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, co
   SMSM_LAUNCH_CHECK("k_is_sched");
   int cl;
   TermFn fn = term_fn(C, &cl);
-  const int chunk = rat_cap(C);
+  const int chunk = scratch_cap(P);
   for (int l0 = 0; l0 < LD; l0 += chunk) {
     const int n = LD - l0 < chunk ? LD - l0 : chunk;
     cudaLaunchConfig_t cfg = {};
@@ -647,8 +630,8 @@ smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, co
     cfg.attrs = at;
     cfg.numAttrs = 1;
     SMSM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, (const float2*)A, (const IsParam*)P->is_prm, (const IsRow*)P->is_tab,
-                                     P->is_part, C, nb, l0));
-    k_is_sum<<<dim3(nblk, n), RB * RB, 0, s>>>(P->is_part, P->Wf, P->is_prm, C, nblk, l0);
+                                     P->scratch, C, nb, l0));
+    k_is_sum<<<dim3(nblk, n), RB * RB, 0, s>>>(P->scratch, P->Wf, P->is_prm, C, nblk, l0);
     SMSM_LAUNCH_CHECK("k_is_sum");
   }
   if (T) T->end(SMSM_STAGE_EIG);

@@ -37,6 +37,26 @@ int vec_blocks(const smsm_plan_s* P) {
   return (int)b;
 }
 
+// Scratch of the Gram and the weight step (which follow one another in a lane), per matrix.  Launches take
+// at most scratch_cap matrices, 96 MB; the buffer has room for every matrix of the plan or, when
+// that is more, one launch's room per lane.
+static size_t scratch_per(const smsm_plan_s* P) {
+  const size_t a = invsqrt_per(P), b = gram_lag_per(P);
+  return a > b ? a : b;
+}
+int scratch_cap(const smsm_plan_s* P) {
+  const size_t n = (size_t)96 * 1024 * 1024 / (scratch_per(P) * sizeof(float2));
+  return n < 1 ? 1 : (int)(n < 4096 ? n : 4096);
+}
+size_t scratch_count(const smsm_plan_s* P) {
+  const size_t cap = scratch_cap(P);
+  return scratch_per(P) * ((size_t)P->LD <= cap ? (size_t)P->LD : cap * SMSM_MAX_LANES);
+}
+static size_t scratch_offset(const smsm_plan_s* P, int d0, int lane) {
+  const size_t cap = scratch_cap(P);
+  return scratch_per(P) * ((size_t)P->LD <= cap ? (size_t)d0 * P->L : cap * lane);
+}
+
 // Sum of partial arrays a[0..na) + b[0..nb) in a fixed order; every thread
 // returns the same value.  `red` is VEC_THREADS doubles of shared memory.
 __device__ double sum_parts(const double* __restrict__ a, int na, const double* __restrict__ b, int nb, double* red) {
@@ -304,7 +324,7 @@ static smsm_plan_s lane_view(const smsm_plan_s* P, int d0, int nd, int lane) {
   v.is_lmax += dd * L;
   v.is_prm += dd * L;
   v.is_flag += dd * L;
-  v.is_part += invsqrt_part_offset(P, d0, lane);
+  v.scratch += scratch_offset(P, d0, lane);
   v.Gpart += cc * P->gram_nkx;
   v.eig += dd * L * Cp;
   v.sweeps += dd * L;
@@ -356,7 +376,8 @@ static smsm_status enqueue_outer(smsm_plan_s* P, const smsm_params* prm, int k, 
   double* rr1 = P->part_rr + (size_t)SMSM_PART_MAX * D;
   const dim3 vg(nvb, D);
   T->begin(SMSM_STAGE_GRAM);
-  if ((st = launch_gram(P, P->xs, P->G64, s))) return st;
+  if ((st = gram_lag_supported(P) ? launch_gram_lag(P, P->xs, P->G64, s) : launch_gram(P, P->xs, P->G64, s)))
+    return st;
   T->end(SMSM_STAGE_GRAM);
   if (eig_wait) SMSM_CUDA_TRY(cudaStreamWaitEvent(s, eig_wait, 0));
   if ((st = launch_eig_weights(P, P->G64, k, prm, s, T))) return st;

@@ -1,7 +1,8 @@
-"""GPU parity of the IRLS weights formed without an eigen-decomposition (csrc/invsqrt.cu).
+"""GPU parity of the solve's FP32 Gram (csrc/gram_lag.cu) and of the IRLS weights formed without an
+eigen-decomposition (csrc/invsqrt.cu).
 
-W = (G + eps I)^(-1/2) is not an output, so it is tested through a short solve against the FP64
-oracle, at the block edges of the kernel: one 16 x 16 block, a ragged last block, the most blocks of one
+Neither is an output, so they are tested through a short solve against the FP64
+oracle, at the edges of the kernels' tiles: one 16 x 16 block, a ragged last block, the most blocks of one
 CTA (C = 192), the first and last sizes of the four-CTA form (C = 196, 294).  Tolerance: the FP32
 whole-solve bar of test_gpu_parity.py (2e-5 per slice), which the eigensolver's weights are held to.
 """
@@ -49,6 +50,11 @@ def worst(x, ref):
     (1, 3, 48, 8),    # C = 192: 78 blocks on one CTA
     (1, 4, 32, 7),    # C = 196: 91 blocks on four CTAs, ragged
     (1, 6, 48, 7),    # C = 294: 190 blocks on four CTAs
+    (1, 1, 16, 8),    # Gram: half a row tile, a core of two rows and columns
+    (2, 2, 36, 2),    # Gram: ragged second row tile, 3 lags
+    (1, 1, 24, 12),   # Gram: 23 lags, one shot per task
+    (1, 2, 48, 10),   # Gram: 19 lags, one shot per task, two shots
+    (3, 3, 96, 1),    # Gram: no edges, odd shot count
 ])
 def test_solve_parity_at_block_edges(smsm, L, Ns, N, r):
     g, y = problem(L, Ns, 6, N, 3)

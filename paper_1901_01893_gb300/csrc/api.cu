@@ -338,6 +338,7 @@ extern "C" smsm_status smsm_plan(smsm_plan_t* out, int mb, int shots, int coils,
   if (!st) st = gram_lag_init_attrs(P);
   if (!st) st = operators_init_attrs();
   if (!st) st = colfast_init_attrs();
+  if (!st) st = colwarp_init_attrs();
   if (!st) st = alias_init_attrs();
   if (!st) st = band_init_attrs(P);
   if (!st) st = gram_tc_init_attrs();

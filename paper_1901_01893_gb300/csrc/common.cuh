@@ -280,6 +280,11 @@ struct ColArgs {
 smsm_status launch_col_fast(const smsm_plan_s* P, const ColArgs& a, cudaStream_t s);
 smsm_status colfast_init_attrs();
 
+// colwarp.cu: the coil loop of A, A^H and the per-coil A^H A a warp at a time; SMSM_ERR_ARG when the
+// geometry has no such kernel
+smsm_status launch_col_warp(const smsm_plan_s* P, int mode, int with_phase, const ColArgs& a, cudaStream_t s);
+smsm_status colwarp_init_attrs();
+
 smsm_status launch_col(const smsm_plan_s* P, int mode, int with_phase, const float2* in, float2* out,
                        const float2* phaseT, const float2* multT, float lambda, double* dot_part,
                        cudaStream_t s);

@@ -546,9 +546,10 @@ smsm_status launch_col(const smsm_plan_s* P, int mode, int with_phase, const flo
   a.dot_part = dot_part;
   a.errflag = P->devflag;
   if (mode == COL_NORMAL && !with_phase && P->alias) return launch_col_alias(P, a, s);
-  if (mode == COL_NORMAL && !with_phase && !(P->flags & SMSM_FLAG_GENERIC_KERNELS)) {
-    smsm_status fst = launch_col_fast(P, a, s);
-    if (fst != SMSM_ERR_ARG) return fst;  // SMSM_ERR_ARG: no fast path for this geometry
+  if (!(P->flags & SMSM_FLAG_GENERIC_KERNELS)) {  // SMSM_ERR_ARG: no such kernel for this geometry
+    smsm_status fst = launch_col_warp(P, mode, with_phase, a, s);
+    if (fst == SMSM_ERR_ARG && mode == COL_NORMAL && !with_phase) fst = launch_col_fast(P, a, s);
+    if (fst != SMSM_ERR_ARG) return fst;
   }
   size_t sm = col_smem(P);
   if (sm > 200 * 1024) {

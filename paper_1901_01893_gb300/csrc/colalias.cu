@@ -75,7 +75,8 @@ __device__ __forceinline__ bool alias_wait(uint64_t* mbar, uint32_t parity) {
 // every shot of its pixel row, and (up to 5 shots) it fetches the slice's
 // Ns(Ns+1)/2 multiplier entries (the Hermitian upper triangle) together, before
 // the class products.
-template <int L, int NS>
+// CLS = false: no class products (A^H A left out), the periodic penalty alone.
+template <int L, int NS, bool CLS>
 __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __restrict__ corr,
                                                    const float2* __restrict__ ash, int sh, int tpy) {
   constexpr int B = L * NS;
@@ -108,7 +109,8 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
     for (int b = 0; b < B; ++b) tma_bulk_g2s(img + b * N, gin + (size_t)b * NN + (size_t)x * N, row_bytes, &bar[0]);
   }
   for (int e = tid; e < N; e += nt) sTwN[e] = a.twN[e];
-  for (int e = tid; e < NS * NS; e += nt) sAsh[e] = ash[e];
+  if (CLS)
+    for (int e = tid; e < NS * NS; e += nt) sAsh[e] = ash[e];
   const bool own = tid < N * tpy;
   const int y = tid % N, bsub = own ? tid / N : B;
   const float sy = sgn_par(y);
@@ -146,14 +148,17 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
     for (int b = bsub; b < B; b += tpy) img[b * N + y] = cscale(R[b * N + y], sc);
   }
   __syncthreads();
+  if constexpr (CLS) {
 #pragma unroll
-  for (int l = 0; l < L; ++l) {
-    int i0 = (bsub - l * NS) % tpy;
-    if (i0 < 0) i0 += tpy;
-    if (!own) i0 = NS;
-    for (int i = i0; i < NS; i += tpy) ph[(l * NS + i) * N + y] = cmul(sAsh[i * NS + kl[l]], img[(l * NS + i) * N + y]);
+    for (int l = 0; l < L; ++l) {
+      int i0 = (bsub - l * NS) % tpy;
+      if (i0 < 0) i0 += tpy;
+      if (!own) i0 = NS;
+      for (int i = i0; i < NS; i += tpy)
+        ph[(l * NS + i) * N + y] = cmul(sAsh[i * NS + kl[l]], img[(l * NS + i) * N + y]);
+    }
+    __syncthreads();
   }
-  __syncthreads();
 
   const float inv_ns = 1.f / (float)NS;
   const float2* cx = corr + (size_t)x * M * B * B;
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
   for (int l = 0; l < L; ++l) {
     float2 c[B];  // row (l, t) of this pixel's class matrix, shared by every shot
     const float2* crow = cx + (size_t)(l * NS + t) * B * M + zl[l];
-    if (own) {
+    if (CLS && own) {
 #pragma unroll
       for (int ap = 0; ap < B; ++ap) c[ap] = __ldg(crow + (size_t)ap * M);
     }
@@ -171,14 +176,17 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
     // output shot i of slice l: class product, plus lambda q (q = sum_j m_ij img_j)
     auto emit = [&](int i, float2 q) {
       const int b = l * NS + i;
-      float2 s = cmk(0.f, 0.f);
+      float2 acc = cmk(0.f, 0.f);
+      if constexpr (CLS) {
+        float2 s = cmk(0.f, 0.f);
 #pragma unroll
-      for (int lp = 0; lp < L; ++lp) {
-        const float2* prow = ph + (lp * NS + i) * N + bs[l][lp];
+        for (int lp = 0; lp < L; ++lp) {
+          const float2* prow = ph + (lp * NS + i) * N + bs[l][lp];
 #pragma unroll
-        for (int tp = 0; tp < NS; ++tp) cfma(s, c[lp * NS + tp], prow[tp * M]);
+          for (int tp = 0; tp < NS; ++tp) cfma(s, c[lp * NS + tp], prow[tp * M]);
+        }
+        acc = cscale(cmulcj(sAsh[i * NS + kl[l]], s), inv_ns);
       }
-      float2 acc = cscale(cmulcj(sAsh[i * NS + kl[l]], s), inv_ns);
       const float2 v = img[b * N + y];
       if (pen) {
         acc.x = fmaf(a.lambda, q.x, acc.x);
@@ -239,9 +247,11 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
 
 typedef void (*ColAliasFn)(ColArgs, const float2*, const float2*, int, int);
 
-#define CA_NS(L) {k_col_alias<L, 1>, k_col_alias<L, 2>, k_col_alias<L, 3>, k_col_alias<L, 4>, \
-                  k_col_alias<L, 5>, k_col_alias<L, 6>, k_col_alias<L, 7>, k_col_alias<L, 8>}
-static const ColAliasFn kColAlias[3][8] = {CA_NS(1), CA_NS(2), CA_NS(3)};
+#define CA_NS(L, CLS) {k_col_alias<L, 1, CLS>, k_col_alias<L, 2, CLS>, k_col_alias<L, 3, CLS>, \
+                       k_col_alias<L, 4, CLS>, k_col_alias<L, 5, CLS>, k_col_alias<L, 6, CLS>, \
+                       k_col_alias<L, 7, CLS>, k_col_alias<L, 8, CLS>}
+static const ColAliasFn kColAlias[3][8] = {CA_NS(1, true), CA_NS(2, true), CA_NS(3, true)};
+static const ColAliasFn kColPen[3][8] = {CA_NS(1, false), CA_NS(2, false), CA_NS(3, false)};
 #undef CA_NS
 
 // threads per pixel row: at least 64 threads per CTA (more threads per row measured slower:
@@ -275,6 +285,8 @@ smsm_status alias_init_attrs() {
   for (int l = 0; l < 3; ++l)
     for (int n = 0; n < 8; ++n) {
       cudaError_t e = cudaFuncSetAttribute(kColAlias[l][n], cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kColPen[l][n], cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       if (e != cudaSuccess) {
         smsm_set_error("cudaFuncSetAttribute (aliasing column stage): %s", cudaGetErrorString(e));
         return SMSM_ERR_CUDA;
@@ -286,6 +298,17 @@ smsm_status alias_init_attrs() {
 smsm_status launch_alias_corr(const smsm_plan_s* P, cudaStream_t s) {
   k_alias_corr<<<1024, 256, 0, s>>>(P->sensT, P->acorr, P->L, P->Ns, P->Nc, P->N, P->M, P->N / P->Ldiv);
   SMSM_LAUNCH_CHECK("k_alias_corr");
+  return SMSM_OK;
+}
+
+// The periodic penalty alone (COL_PEN) by the same kernel without its classes (k_col<COL_PEN> 137 us, this 62 us:
+// 256 x 256, 48 slice-shots); SMSM_ERR_ARG when the geometry is outside its range
+smsm_status launch_col_pen(const smsm_plan_s* P, const ColArgs& a, cudaStream_t s) {
+  const int B = P->L * P->Ns;
+  if (P->L > 3 || P->Ns > 8 || alias_threads(P->N, B) > 512 || alias_smem(P) > 200 * 1024) return SMSM_ERR_ARG;
+  kColPen[P->L - 1][P->Ns - 1]<<<dim3(P->N, P->D), alias_threads(P->N, B), alias_smem(P), s>>>(
+      a, nullptr, nullptr, 0, alias_tpy(P->N, B));
+  SMSM_LAUNCH_CHECK("k_col_alias (penalty)");
   return SMSM_OK;
 }
 

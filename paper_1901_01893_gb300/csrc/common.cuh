@@ -294,6 +294,7 @@ size_t alias_corr_count(const smsm_plan_s* P);
 smsm_status alias_init_attrs();
 smsm_status launch_alias_corr(const smsm_plan_s* P, cudaStream_t s);
 smsm_status launch_col_alias(const smsm_plan_s* P, const ColArgs& a, cudaStream_t s);
+smsm_status launch_col_pen(const smsm_plan_s* P, const ColArgs& a, cudaStream_t s);
 // hankel.cu
 smsm_status launch_gram(const smsm_plan_s* P, const float2* x, double2* G, cudaStream_t s);
 // gram_tc.cu

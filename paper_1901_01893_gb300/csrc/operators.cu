@@ -547,7 +547,7 @@ smsm_status launch_col(const smsm_plan_s* P, int mode, int with_phase, const flo
   a.errflag = P->devflag;
   if (mode == COL_NORMAL && !with_phase && P->alias) return launch_col_alias(P, a, s);
   if (!(P->flags & SMSM_FLAG_GENERIC_KERNELS)) {  // SMSM_ERR_ARG: no such kernel for this geometry
-    smsm_status fst = launch_col_warp(P, mode, with_phase, a, s);
+    smsm_status fst = mode == COL_PEN ? launch_col_pen(P, a, s) : launch_col_warp(P, mode, with_phase, a, s);
     if (fst == SMSM_ERR_ARG && mode == COL_NORMAL && !with_phase) fst = launch_col_fast(P, a, s);
     if (fst != SMSM_ERR_ARG) return fst;
   }

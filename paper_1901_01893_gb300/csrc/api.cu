@@ -108,6 +108,10 @@ static void free_plan(smsm_plan_s* P) {
     if (P->lane_s[k]) cudaStreamDestroy(P->lane_s[k]);
   for (int k = 0; k < 2 * SMSM_MAX_LANES + 1; ++k)
     if (P->lane_ev[k]) cudaEventDestroy(P->lane_ev[k]);
+  for (int k = 0; k < SMSM_MAX_LANES; ++k)
+    if (P->band_s[k]) cudaStreamDestroy(P->band_s[k]);
+  for (int k = 0; k < 2 * SMSM_MAX_LANES; ++k)
+    if (P->band_ev[k]) cudaEventDestroy(P->band_ev[k]);
   if (P->ev0) cudaEventDestroy(P->ev0);
   if (P->ev1) cudaEventDestroy(P->ev1);
   free(P);
@@ -279,6 +283,7 @@ extern "C" smsm_status smsm_plan(smsm_plan_t* out, int mb, int shots, int coils,
     free_plan(P);
     return st;
   }
+  P->band_px = band_px(P);
   P->nvb = vec_blocks(P);  // fixed for the plan: lanes (sub-batches) reduce in the same order
   if (band_blocks(P) > SMSM_PART_MAX || vec_blocks(P) > SMSM_PART_MAX) {
     free_plan(P);
@@ -358,6 +363,10 @@ extern "C" smsm_status smsm_plan(smsm_plan_t* out, int mb, int shots, int coils,
     cudaError_t e = cudaStreamCreateWithFlags(&P->cap_stream, cudaStreamNonBlocking);
     for (int k = 1; k < SMSM_MAX_LANES && e == cudaSuccess; ++k)
       e = cudaStreamCreateWithFlags(&P->lane_s[k], cudaStreamNonBlocking);
+    for (int k = 0; k < SMSM_MAX_LANES && k < D && e == cudaSuccess; ++k)
+      e = cudaStreamCreateWithFlags(&P->band_s[k], cudaStreamNonBlocking);
+    for (int k = 0; k < 2 * SMSM_MAX_LANES && e == cudaSuccess; ++k)
+      e = cudaEventCreateWithFlags(&P->band_ev[k], cudaEventDisableTiming);
     for (int k = 0; k < 2 * SMSM_MAX_LANES + 1 && e == cudaSuccess; ++k)
       e = cudaEventCreateWithFlags(&P->lane_ev[k], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreate(&P->ev0);
@@ -496,7 +505,7 @@ extern "C" smsm_status smsm_apply_filters(smsm_plan_t plan, const void* W, const
   if ((st = launch_rowfft_out_T(plan, (const float2*)x, plan->hA, B, plan->N, 1, s))) return st;
   if ((st = launch_col(plan, COL_PEN, 0, plan->hA, plan->hB, nullptr, plan->multT, 1.f, nullptr, s))) return st;
   if ((st = launch_rowfft_in_T(plan, plan->hB, (float2*)out, B, plan->N, 0, s))) return st;
-  return launch_band(plan, (const float2*)x, (float2*)out, 1.f, nullptr, s);
+  return launch_band(plan, (const float2*)x, (float2*)out, 1.f, nullptr, 1, s);
 }
 
 extern "C" smsm_status smsm_fft2c(smsm_plan_t plan, const void* in, void* out, int count, int inverse, void* stream) {

@@ -202,16 +202,17 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
   }
 
   // partial of Re<img, acc> (Parseval: equals Re<p, q> in k-space)
-  double dsum = 0.0;
+  float ds = 0.f;  // FP32 over this lane's few pixels, FP64 from there on
 #pragma unroll
   for (int l = 0; l < L; ++l)
 #pragma unroll
     for (int k = 0; k < NK; ++k) {
       const int y = lane + 32 * k;
       const float2 u = img[(l * Ns + i) * N + y];
-      dsum += (double)u.x * acc[l][k].x + (double)u.y * acc[l][k].y;
+      ds = fmaf(u.x, acc[l][k].x, fmaf(u.y, acc[l][k].y, ds));
       tmp[(l * Ns + i) * N + y] = cscale(acc[l][k], sgn_par(y));
     }
+  double dsum = ds;
   for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
   if (lane == 0) red[warp] = dsum;
   __syncthreads();

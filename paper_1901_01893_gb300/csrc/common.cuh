@@ -38,6 +38,13 @@ __device__ __forceinline__ void cfmacj(float2& acc, float2 a, float2 b) {
   acc.y = fmaf(-a.y, b.x, acc.y);
 }
 
+// s + c += v, the rounding of s kept in c
+__device__ __forceinline__ void add2(float& s, float& c, float v) {
+  const float t = s + v, z = t - s;
+  c += (s - (t - z)) + (v - z);
+  s = t;
+}
+
 // asynchronous 8-byte global -> shared copy (completes at cp_async_wait_all)
 // Periodic penalty multiplier m_ii'[x][y] of one (direction, slice).  It is
 // Hermitian in the shot pair (wt_ii'[d] = conj(wt_i'i[-d]) because W is), so only
@@ -131,6 +138,7 @@ struct smsm_plan_s {
   float2* ash;    // [Ns][Ns]: exp(-2 pi j (i - N/2) q / Ns)
   int* devflag;   // device error flag raised by bounded waits (SMSM_ERR_TIMEOUT)
   int LD;  // D * L: number of (direction, slice) Hankel matrices
+  int band_px;  // pixels per lane of the border band
   int nvb; // CTAs per direction of the CG vector kernels (fixed at plan creation)
   int nband;  // pixels within r-1 of an edge
   int dev;
@@ -173,6 +181,9 @@ struct smsm_plan_s {
   unsigned graph_gen;  // bumped whenever the captured solve is dropped (group launches re-check it)
   cudaStream_t cap_stream;
   cudaStream_t lane_s[SMSM_MAX_LANES];  // capture streams of lanes 1.. (lane 0 captures on cap_stream)
+  cudaStream_t band_s[SMSM_MAX_LANES];  // capture streams of the lanes' border bands
+  cudaEvent_t band_ev[2 * SMSM_MAX_LANES];  // fork and join of a lane's band
+  int lane;  // the lane a sub-batch view is solved as
   cudaEvent_t lane_ev[2 * SMSM_MAX_LANES + 1];  // fork, per-lane join and eigen-step events
   smsm_params gparams;
   int has_graph;
@@ -251,8 +262,9 @@ struct Timer {
 smsm_status launch_transpose(const float2* in, float2* out, int nb, int rows, int cols, cudaStream_t s);
 smsm_status launch_rowfft_out_T(const smsm_plan_s* P, const float2* in, float2* out, int nb, int rows,
                                 int inverse, cudaStream_t s);
+// band > 0: added to what out holds at the pixels within band of an edge (rows x N images)
 smsm_status launch_rowfft_in_T(const smsm_plan_s* P, const float2* in, float2* out, int nb, int rows,
-                               int inverse, cudaStream_t s);
+                               int inverse, cudaStream_t s, int band = 0);
 // inverse row FFT of p (N rows per image) with the CG update p = r + beta p fused in
 smsm_status launch_rowfft_out_T_cgp(const smsm_plan_s* P, float2* p, const float2* r, float2* out, int nb,
                                     const double* rr_new, const double* rr_old, int nrr, cudaStream_t s);
@@ -310,8 +322,10 @@ size_t gram_lag_per(const smsm_plan_s* P);
 smsm_status gram_lag_init_attrs(const smsm_plan_s* P);
 smsm_status launch_gram_lag(const smsm_plan_s* P, const float2* x, double2* G, cudaStream_t s);
 smsm_status launch_filters(const smsm_plan_s* P, const float2* W, cudaStream_t s);
-smsm_status launch_band(const smsm_plan_s* P, const float2* x, float2* out, float scale, double* dot_part,
+smsm_status launch_band(const smsm_plan_s* P, const float2* x, float2* out, float scale, double* dot_part, int add,
                         cudaStream_t s);
+int band_width(const smsm_plan_s* P);
+int band_px(const smsm_plan_s* P);
 smsm_status launch_w_from_c128(const smsm_plan_s* P, const double2* W64, float2* W, cudaStream_t s);
 // eig.cu
 void solver_drop_graph(smsm_plan_s* P);

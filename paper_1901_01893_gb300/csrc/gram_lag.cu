@@ -201,13 +201,6 @@ __global__ void __launch_bounds__(32 * LAG_MAXW) k_lag(const float2* __restrict_
   }
 }
 
-// s + c += v, the rounding of s kept in c
-__device__ __forceinline__ void add2(float& s, float& c, float v) {
-  const float t = s + v, z = t - s;
-  c += (s - (t - z)) + (v - z);
-  s = t;
-}
-
 // One warp per (matrix, task, p_y, p_x), lanes over the NJ (2r-1) lags of the task.
 __global__ void __launch_bounds__(256) k_lag_sum(const float2* __restrict__ part, double2* __restrict__ G, int Ns, int r,
                                                  int C, int nj, int ntask, int nty, int l0) {

@@ -321,21 +321,21 @@ smsm_status launch_filters(const smsm_plan_s* P, const float2* W, cudaStream_t s
 // taps once per CTA; the corner pixels each have their own class and are
 // summed by k_band_corner.
 // ---------------------------------------------------------------------------
-#define BAND_P 2                  // pixels per thread
-#define BAND_TX (32 * BAND_P)     // pixels per strip line per CTA
-
-// One CTA = one chunk of BAND_TX pixels of one line of one strip; warp j sums
+// One CTA = one chunk of 32 PX pixels of one line of one strip; warp j sums
 // the taps of input shot j for every output shot; the NS partials of each
-// (pixel, output shot) are then added in a fixed order (deterministic).  The
-// line's window of x (2r-1 lines across, BAND_TX + 2r-2 along, periodically
-// wrapped) is staged in shared memory as [shot][across][along] for both
-// orientations, and so are the line's taps [j][d][i] (read as broadcasts); both
-// with asynchronous copies, all in flight at once.  Lane q owns the pixels
-// q + 32 p (p < BAND_P), so the window reads of a warp are consecutive.
-template <int NS>
+// (pixel, output shot) are then added in a fixed order (deterministic).  Only taps whose patches
+// leave the image correct anything: on line c of a low strip those across offsets up to 2r-3-c, on a
+// high one from r-1-c on (six to ten of eleven at r = 6).  The line's window of x (those lines across,
+// 32 PX + 2r-2 along, periodically wrapped) is staged in shared memory for both orientations, and so are the
+// line's taps [j][d][i] (read as broadcasts); both with asynchronous copies, all in flight at once.
+// Lane q owns the PX consecutive pixels from PX q on, their window turning through PX registers: one window load
+// and one set of taps per PX NS complex multiply-adds.  A window row is stored as PX planes (element n in plane n
+// mod PX), so that a warp's loads are consecutive.  FMA-bound; PX from band_px.
+template <int NS, int PX>
 __global__ void __launch_bounds__(32 * NS) k_band(const float2* __restrict__ x, float2* __restrict__ out,
                                                   const float2* __restrict__ dcls, int L, int N, int r, float scale,
-                                                  double* __restrict__ dot_part) {
+                                                  double* __restrict__ dot_part, int add) {
+  constexpr int TX = 32 * PX;
   extern __shared__ __align__(16) float2 bsm[];
   __shared__ double red[8];
   const int R2 = 2 * r - 1, w = r - 1;
@@ -344,14 +344,15 @@ __global__ void __launch_bounds__(32 * NS) k_band(const float2* __restrict__ x, 
   const int d = lf / L, l = lf - d * L;
   const int horiz = strip < 2;
   const int lo = (strip == 0 || strip == 2);
-  const int nchunk = (N - 2 * w + BAND_TX - 1) / BAND_TX;
+  const int nchunk = (N - 2 * w + TX - 1) / TX;
   const int line = blockIdx.x / nchunk, chunk = blockIdx.x - line * nchunk;
   const int tid = threadIdx.x, j = tid >> 5, lane = tid & 31;
   const int nt = blockDim.x;
-  const int Wl = BAND_TX + R2 - 1;
-  const int start = w + chunk * BAND_TX;  // first pixel along the line
+  const int PL = (TX + R2 - 1 + PX - 1) / PX, Wl = PX * PL;  // plane, window row
+  const int start = w + chunk * TX;  // first pixel along the line
   const int limit = N - w;
   const int fixed = (lo ? 0 : N - w) + line;
+  const int a0 = lo ? 0 : w - line, a1 = lo ? 2 * r - 2 - line : R2;  // across offsets [a0, a1)
   const size_t NN = (size_t)N * N;
   const float2* xl = x + (size_t)lf * NS * NN;
   const int ntap = NS * R2 * R2 * NS;  // taps of one class
@@ -359,90 +360,90 @@ __global__ void __launch_bounds__(32 * NS) k_band(const float2* __restrict__ x, 
   const int clsline = horiz ? cfix * R2 + (r - 1) : (r - 1) * R2 + cfix;
   const float2* tl = dcls + ((size_t)lf * R2 * R2 + clsline) * ntap;
   float2* tsm = bsm;                               // [NS (j)][R2*R2][NS (i)]
-  float2* xs = tsm + ((ntap + 1) & ~1);            // [NS][R2][Wl]
-  float2* part = xs;                               // [NS (j)][BAND_TX][NS (i)], after the window is used
+  float2* xs = tsm + ((ntap + 1) & ~1);            // [NS][R2][PX][PL]
+  float2* part = xs;                               // [NS (j)][TX][NS (i)], after the window is used
   for (int e = tid; e < ntap; e += nt) cp_async8(tsm + e, tl + e);
   // window rows (shot jj, across aa): one warp per row, lanes along the line.  Along the
-  // line only [start - w, min(start + BAND_TX, limit) + w) is read by kept pixels: all of
+  // line only [start - w, min(start + TX, limit) + w) is read by kept pixels: all of
   // it inside the image (the rest of the row is never written and only feeds discarded
   // pixels); across the line the window wraps periodically.
-  const int Wv = min(Wl, limit - start + 2 * w);
-  for (int row = j; row < NS * R2; row += nt >> 5) {
-    const int jj = row / R2, aa = row - jj * R2;
-    float2* dst = xs + (size_t)row * Wl;
-    if (horiz) {
-      int gy = fixed + aa - w;
-      gy = gy < 0 ? gy + N : (gy >= N ? gy - N : gy);
-      const float2* src = xl + (size_t)jj * NN + (size_t)gy * N + (start - w);
-      for (int u = lane; u < Wv; u += 32) cp_async8(dst + u, src + u);
-    } else {
-      int gx = fixed + aa - w;
-      gx = gx < 0 ? gx + N : (gx >= N ? gx - N : gx);
-      const float2* src = xl + (size_t)jj * NN + (size_t)(start - w) * N + gx;
-      for (int u = lane; u < Wv; u += 32) cp_async8(dst + u, src + (size_t)u * N);
-    }
+  const int Wv = min(TX + R2 - 1, limit - start + 2 * w);
+  for (int row = j; row < NS * (a1 - a0); row += nt >> 5) {
+    const int jj = row / (a1 - a0), aa = a0 + row - jj * (a1 - a0);
+    float2* dst = xs + (size_t)(jj * R2 + aa) * Wl;
+    int g = fixed + aa - w;
+    g = g < 0 ? g + N : (g >= N ? g - N : g);
+    const float2* src = xl + (size_t)jj * NN + (horiz ? (size_t)g * N + (start - w) : (size_t)(start - w) * N + g);
+    const size_t step = horiz ? 1 : N;
+    for (int u = lane; u < Wv; u += 32) cp_async8(dst + (u % PX) * PL + u / PX, src + u * step);
   }
   cp_async_wait_all();
   __syncthreads();
-  float2 acc[BAND_P][NS];
+  float2 acc[PX][NS];
 #pragma unroll
-  for (int p = 0; p < BAND_P; ++p)
+  for (int p = 0; p < PX; ++p)
 #pragma unroll
     for (int i = 0; i < NS; ++i) acc[p][i] = cmk(0.f, 0.f);
   {
     const float2* taps = tsm + (size_t)j * R2 * R2 * NS;
     // tap (aa, bb) of the line is d = aa R2 + bb (horizontal strips) or bb R2 + aa
     const int tstep = (horiz ? 1 : R2) * NS;
-    for (int aa = 0; aa < R2; ++aa) {
+    for (int aa = a0; aa < a1; ++aa) {
       const float2* xr = xs + ((size_t)j * R2 + aa) * Wl + lane;
-      const float2* tp0 = taps + (size_t)(horiz ? aa * R2 : aa) * NS;
-#pragma unroll 4
-      for (int bb = 0; bb < R2; ++bb) {
-        const float2* tp = tp0 + bb * tstep;
-        float2 tv[NS];
-        if (NS % 2 == 0 && (ntap % 2 == 0)) {
+      const float2* tp = taps + (size_t)(horiz ? aa * R2 : aa) * NS;
+      float2 win[PX];
 #pragma unroll
-          for (int i = 0; i + 1 < NS; i += 2) {
-            const float4 t4 = *reinterpret_cast<const float4*>(tp + i);
-            tv[i] = cmk(t4.x, t4.y);
-            tv[i + 1] = cmk(t4.z, t4.w);
+      for (int p = 0; p + 1 < PX; ++p) win[p] = xr[p * PL];
+      for (int b0 = 0; b0 < R2; b0 += PX, xr += 1) {
+#pragma unroll
+        for (int u = 0; u < PX; ++u) {
+          if (b0 + u >= R2) break;
+          win[(u + PX - 1) % PX] = xr[((u + PX - 1) % PX) * PL + (u + PX - 1) / PX];
+          float2 tv[NS];
+          if (NS % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i + 1 < NS; i += 2) {
+              const float4 t4 = *reinterpret_cast<const float4*>(tp + i);
+              tv[i] = cmk(t4.x, t4.y);
+              tv[i + 1] = cmk(t4.z, t4.w);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < NS; ++i) tv[i] = tp[i];
           }
-        } else {
+          tp += tstep;
 #pragma unroll
-          for (int i = 0; i < NS; ++i) tv[i] = tp[i];
-        }
+          for (int p = 0; p < PX; ++p)
 #pragma unroll
-        for (int p = 0; p < BAND_P; ++p) {
-          const float2 xv = xr[32 * p + bb];
-#pragma unroll
-          for (int i = 0; i < NS; ++i) cfma(acc[p][i], tv[i], xv);
+            for (int i = 0; i < NS; ++i) cfma(acc[p][i], tv[i], win[(u + p) % PX]);
         }
       }
     }
   }
   __syncthreads();  // the window is no longer read: part takes its place
 #pragma unroll
-  for (int p = 0; p < BAND_P; ++p)
+  for (int p = 0; p < PX; ++p)
 #pragma unroll
-    for (int i = 0; i < NS; ++i) part[((size_t)j * BAND_TX + lane + 32 * p) * NS + i] = acc[p][i];
+    for (int i = 0; i < NS; ++i) part[((size_t)j * TX + lane * PX + p) * NS + i] = acc[p][i];
   __syncthreads();
-  double dsum = 0.0;
-  for (int t = tid; t < BAND_TX * NS; t += nt) {
+  float ds = 0.f;  // FP32 over this thread's few pixels, FP64 from there on
+  for (int t = tid; t < TX * NS; t += nt) {
     const int pu = t / NS, i = t - pu * NS;
     const int pos = start + pu;
     if (pos >= limit) continue;
     float2 sacc = part[(size_t)pu * NS + i];
-    for (int jj = 1; jj < NS; ++jj) sacc = cadd(sacc, part[((size_t)jj * BAND_TX + pu) * NS + i]);
+    for (int jj = 1; jj < NS; ++jj) sacc = cadd(sacc, part[((size_t)jj * TX + pu) * NS + i]);
     const int ny = horiz ? fixed : pos, nx = horiz ? pos : fixed;
     const size_t o = ((size_t)lf * NS + i) * NN + (size_t)ny * N + nx;
     const float2 c = cscale(sacc, scale);
-    out[o] = cadd(out[o], c);
+    out[o] = add ? cadd(out[o], c) : c;
     if (dot_part) {
       const float2 xv = xl[(size_t)i * NN + (size_t)ny * N + nx];
-      dsum += (double)xv.x * c.x + (double)xv.y * c.y;
+      ds = fmaf(xv.x, c.x, fmaf(xv.y, c.y, ds));
     }
   }
   if (dot_part) {
+    double dsum = ds;
     for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
     if (lane == 0) red[j] = dsum;
     __syncthreads();
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(BAND_CORNER_THREADS) k_band_corner(const float
                                                                      float2* __restrict__ out,
                                                                      const float2* __restrict__ dcls, int L, int Ns,
                                                                      int N, int r, float scale,
-                                                                     double* __restrict__ dot_part, int part_base) {
+                                                                     double* __restrict__ dot_part, int part_base, int add) {
   extern __shared__ __align__(16) float2 csm[];
   const int R2 = 2 * r - 1, w = r - 1, RR = R2 * R2;
   const int pix = blockIdx.x;     // py * w + px
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(BAND_CORNER_THREADS) k_band_corner(const float
       for (int k = 0; k < Ns * nc; ++k) sacc = cadd(sacc, part[(size_t)i * Ns * nc + k]);
       const size_t o = ((size_t)lf * Ns + i) * NN + (size_t)ny * N + nx;
       const float2 cc = cscale(sacc, scale);
-      out[o] = cadd(out[o], cc);
+      out[o] = add ? cadd(out[o], cc) : cc;
       if (dot_part) {
         const float2 xv = xl[(size_t)i * NN + (size_t)ny * N + nx];
         dsum += (double)xv.x * cc.x + (double)xv.y * cc.y;
@@ -531,8 +532,33 @@ static size_t band_corner_smem(const smsm_plan_s* P) {
   return (Ns * R2 * R2 * Ns + Ns * R2 * R2 + npair * nc) * sizeof(float2);
 }
 
+static size_t band_smem_px(const smsm_plan_s* P, int px) {
+  const int R2 = P->R2, Ns = P->Ns, tx = 32 * px;
+  const size_t ntap = (size_t)Ns * R2 * R2 * Ns;
+  const size_t win = (size_t)Ns * R2 * px * ((tx + R2 - 1 + px - 1) / px), part = (size_t)Ns * tx * Ns;
+  return (((ntap + 1) & ~(size_t)1) + (win > part ? win : part)) * sizeof(float2);
+}
+
+// Pixels per lane, fixed for the plan (a sub-batch adds its partial sums up the same way): the fewest lanes left
+// over on a line (its N - 2(r-1) pixels in chunks of 32 px), then the most pixels per load; more than two only
+// where two CTAs still fit an SM and the CTAs fill the chip (one 128 x 128 direction: 12 us with two, 14 with four).
+int band_px(const smsm_plan_s* P) {
+  if (P->band_px > 0) return P->band_px;
+  const int n = P->N - 2 * (P->r - 1);
+  int best = 2, least = (n + 63) / 64 * 64;
+  for (int px = 3; px <= 4; ++px) {
+    const int chunks = (n + 32 * px - 1) / (32 * px), len = chunks * 32 * px;
+    if (len <= least && band_smem_px(P, px) <= 110 * 1024 && (long)4 * (P->r - 1) * chunks * P->LD >= 304) {
+      best = px;
+      least = len;
+    }
+  }
+  return best;
+}
+
 static int band_chunks(const smsm_plan_s* P) {
-  return (P->r - 1) * ((P->N - 2 * (P->r - 1) + BAND_TX - 1) / BAND_TX);
+  const int tx = 32 * band_px(P);
+  return (P->r - 1) * ((P->N - 2 * (P->r - 1) + tx - 1) / tx);
 }
 
 // partial sums per direction written by k_band and k_band_corner
@@ -540,25 +566,15 @@ int band_blocks(const smsm_plan_s* P) {
   return (P->r > 1 && !P->periodic) ? P->L * 4 * band_chunks(P) + P->L * 4 * (P->r - 1) * (P->r - 1) : 0;
 }
 
-static size_t band_smem(const smsm_plan_s* P) {
-  const int R2 = P->R2, Ns = P->Ns;
-  const size_t ntap = (size_t)Ns * R2 * R2 * Ns;
-  const size_t win = (size_t)Ns * R2 * (BAND_TX + R2 - 1), part = (size_t)Ns * BAND_TX * Ns;
-  return (((ntap + 1) & ~(size_t)1) + (win > part ? win : part)) * sizeof(float2);
-}
+static size_t band_smem(const smsm_plan_s* P) { return band_smem_px(P, band_px(P)); }
 
-typedef void (*BandFn)(const float2*, float2*, const float2*, int, int, int, float, double*);
+typedef void (*BandFn)(const float2*, float2*, const float2*, int, int, int, float, double*, int);
 static BandFn band_fn(const smsm_plan_s* P) {
-  switch (P->Ns) {
-    case 1: return k_band<1>;
-    case 2: return k_band<2>;
-    case 3: return k_band<3>;
-    case 4: return k_band<4>;
-    case 5: return k_band<5>;
-    case 6: return k_band<6>;
-    case 7: return k_band<7>;
-    default: return k_band<8>;
-  }
+#define BAND_NS(PX) {k_band<1, PX>, k_band<2, PX>, k_band<3, PX>, k_band<4, PX>, \
+                     k_band<5, PX>, k_band<6, PX>, k_band<7, PX>, k_band<8, PX>}
+  static const BandFn fn[3][8] = {BAND_NS(2), BAND_NS(3), BAND_NS(4)};
+#undef BAND_NS
+  return fn[band_px(P) - 2][P->Ns - 1];
 }
 
 smsm_status band_init_attrs(const smsm_plan_s* P) {
@@ -574,18 +590,23 @@ smsm_status band_init_attrs(const smsm_plan_s* P) {
   return SMSM_OK;
 }
 
-smsm_status launch_band(const smsm_plan_s* P, const float2* x, float2* out, float scale, double* dot_part,
+// add != 0: out += the correction; 0: out = the correction at the band's pixels (the x transform that follows adds
+// its result to them: see launch_rowfft_in_T's band)
+smsm_status launch_band(const smsm_plan_s* P, const float2* x, float2* out, float scale, double* dot_part, int add,
                         cudaStream_t s) {
   if (P->r <= 1 || P->periodic) {  // filter 1 or periodic patches: the periodic value is exact
     if (dot_part) SMSM_CUDA_TRY(cudaMemsetAsync(dot_part, 0, sizeof(double) * SMSM_PART_MAX * P->D, s));
     return SMSM_OK;
   }
   dim3 grid(band_chunks(P), 4, P->LD);
-  band_fn(P)<<<grid, 32 * P->Ns, band_smem(P), s>>>(x, out, P->wcls, P->L, P->N, P->r, scale, dot_part);
+  band_fn(P)<<<grid, 32 * P->Ns, band_smem(P), s>>>(x, out, P->wcls, P->L, P->N, P->r, scale, dot_part, add);
   SMSM_LAUNCH_CHECK("k_band");
   // corner pixels: disjoint from the strips, so the two kernels may run in either order
   k_band_corner<<<dim3((P->r - 1) * (P->r - 1), 4, P->LD), BAND_CORNER_THREADS, band_corner_smem(P), s>>>(
-      x, out, P->wcls, P->L, P->Ns, P->N, P->r, scale, dot_part, P->L * 4 * band_chunks(P));
+      x, out, P->wcls, P->L, P->Ns, P->N, P->r, scale, dot_part, P->L * 4 * band_chunks(P), add);
   SMSM_LAUNCH_CHECK("k_band_corner");
   return SMSM_OK;
 }
+
+// width of the band of pixels that launch_band writes
+int band_width(const smsm_plan_s* P) { return P->periodic ? 0 : P->r - 1; }

@@ -238,17 +238,19 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
         q += sq[k];
       }
       // c bounds the largest eigenvalue: row sums or the Frobenius norm (a little above, for rounding)
-      const double eps = eps_s;
-      const double c = 1.0001 * (fmin((double)m, sqrt((double)q)) + eps);
+      // (FP32: A = (G + eps I)/c whatever c is, as long as its parts use the same one)
+      const float eps = (float)eps_s;
+      const float c = 1.0001f * (fminf(m, sqrtf(q)) + eps);
       IsParam p;
-      p.inv_c = (float)(1.0 / c);
-      p.shift = (float)(eps / c);
-      p.wscale = (float)(1.0 / sqrt(c));
+      p.inv_c = 1.f / c;
+      p.shift = eps * p.inv_c;
+      p.wscale = sqrtf(p.inv_c);
       p.q = 0;
       p.n = 0;
-      if (q > 0.f && eps > 0.0 && c / eps <= (double)(1 << IS_MAXQ)) {  // false for NaN too
+      const float cond = c / eps;
+      if (q > 0.f && eps > 0.f && cond <= (float)(1 << IS_MAXQ)) {  // false for NaN too
         int k = 0;
-        while ((double)(1 << k) < c / eps) ++k;
+        while ((float)(1 << k) < cond) ++k;
         p.q = k;
         p.n = tab[k].n;
       }

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) k_rowfft_out_T(const float2* __restrict__
 template <bool INV>
 __global__ void __launch_bounds__(256) k_rowfft_in_T(const float2* __restrict__ in, float2* __restrict__ out,
                                                      int rows, int TY, FftDesc d, const float2* __restrict__ tw,
-                                                     float sN, int vec) {
+                                                     float sN, int vec, int band) {
   extern __shared__ float2 sm[];
   const int N = d.n, ld = N + 1;
   float2* b0 = sm;
@@ -168,12 +168,24 @@ __global__ void __launch_bounds__(256) k_rowfft_in_T(const float2* __restrict__ 
     for (int e = threadIdx.x; e < TY * N / 2; e += blockDim.x) {
       const int f = 2 * e, row = f / N, col = f - row * N;  // col even: signs +, -
       const float2 u = R[row * ld + col], w = R[row * ld + col + 1];
-      dst4[e] = make_float4(sN * u.x, sN * u.y, -sN * w.x, -sN * w.y);
+      float4 v = make_float4(sN * u.x, sN * u.y, -sN * w.x, -sN * w.y);
+      if (band) {
+        const bool edge = r0 + row < band || r0 + row >= rows - band;
+        const bool e0 = edge || col < band || col >= N - band, e1 = edge || col + 1 < band || col + 1 >= N - band;
+        if (e0 || e1) {
+          const float4 o = dst4[e];
+          if (e0) v.x += o.x, v.y += o.y;
+          if (e1) v.z += o.z, v.w += o.w;
+        }
+      }
+      dst4[e] = v;
     }
   } else {
     for (int e = threadIdx.x; e < TY * N; e += blockDim.x) {
       int row = e / N, col = e - row * N;
-      dst[e] = cscale(R[row * ld + col], sN * sgn_par(col));
+      float2 v = cscale(R[row * ld + col], sN * sgn_par(col));
+      if (band && (r0 + row < band || r0 + row >= rows - band || col < band || col >= N - band)) v = cadd(v, dst[e]);
+      dst[e] = v;
     }
   }
 }
@@ -291,15 +303,15 @@ smsm_status launch_rowfft_out_T_cgp(const smsm_plan_s* P, float2* p, const float
 }
 
 smsm_status launch_rowfft_in_T(const smsm_plan_s* P, const float2* in, float2* out, int nb, int rows,
-                               int inverse, cudaStream_t s) {
+                               int inverse, cudaStream_t s, int band) {
   const int TY = pick_ty(rows);
   const int vec = rowfft_vec(in, out);
   dim3 grid(rows / TY, nb);
   size_t sm = rowfft_smem(P->N, TY);
   if (inverse)
-    k_rowfft_in_T<true><<<grid, 256, sm, s>>>(in, out, rows, TY, P->fN, P->twN, P->sN, vec);
+    k_rowfft_in_T<true><<<grid, 256, sm, s>>>(in, out, rows, TY, P->fN, P->twN, P->sN, vec, band);
   else
-    k_rowfft_in_T<false><<<grid, 256, sm, s>>>(in, out, rows, TY, P->fN, P->twN, P->sN, vec);
+    k_rowfft_in_T<false><<<grid, 256, sm, s>>>(in, out, rows, TY, P->fN, P->twN, P->sN, vec, band);
   SMSM_LAUNCH_CHECK("k_rowfft_in_T");
   return SMSM_OK;
 }

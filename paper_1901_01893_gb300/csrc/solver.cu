@@ -270,21 +270,32 @@ static smsm_status normal_pen_timed(smsm_plan_s* P, const float2* v, float2* q, 
     return st;
   }
   if (T) T->end(SMSM_STAGE_ROWFFT_INV);
+  // The border band needs v only: while the solve is captured it is a branch of its own beside the column
+  // stage, and the x transform that follows both adds its result to the band's pixels of q.  (Timed
+  // solves keep one stream, so that a bracket holds its stage alone.)
+  const bool fork = T && !T->mask && lambda != 0.f;
+  cudaStream_t bs = fork ? P->band_s[P->lane] : s;
+  if (lambda != 0.f) {
+    if (fork) {
+      SMSM_CUDA_TRY(cudaEventRecord(P->band_ev[2 * P->lane], s));
+      SMSM_CUDA_TRY(cudaStreamWaitEvent(bs, P->band_ev[2 * P->lane], 0));
+    }
+    if (T) T->begin(SMSM_STAGE_BAND);
+    if ((st = launch_band(P, v, q, lambda, with_dots ? P->part_pq_band : nullptr, 0, bs))) return st;
+    if (T) T->end(SMSM_STAGE_BAND);
+    if (fork) SMSM_CUDA_TRY(cudaEventRecord(P->band_ev[2 * P->lane + 1], bs));
+  } else if (with_dots) {
+    SMSM_CUDA_TRY(cudaMemsetAsync(P->part_pq_band, 0, sizeof(double) * SMSM_PART_MAX * P->D, s));
+  }
   if (T) T->begin(SMSM_STAGE_COLUMN);
   if ((st = launch_col(P, COL_NORMAL, 0, P->hA, P->hB, nullptr, lambda != 0.f ? P->multT : nullptr, lambda,
                        with_dots ? P->part_pq_col : nullptr, s)))
     return st;
   if (T) T->end(SMSM_STAGE_COLUMN);
   if (T) T->begin(SMSM_STAGE_ROWFFT_FWD);
-  if ((st = launch_rowfft_in_T(P, P->hB, q, P->D * B, P->N, 0, s))) return st;
+  if (fork) SMSM_CUDA_TRY(cudaStreamWaitEvent(s, P->band_ev[2 * P->lane + 1], 0));
+  if ((st = launch_rowfft_in_T(P, P->hB, q, P->D * B, P->N, 0, s, lambda != 0.f ? band_width(P) : 0))) return st;
   if (T) T->end(SMSM_STAGE_ROWFFT_FWD);
-  if (lambda != 0.f) {
-    if (T) T->begin(SMSM_STAGE_BAND);
-    if ((st = launch_band(P, v, q, lambda, with_dots ? P->part_pq_band : nullptr, s))) return st;
-    if (T) T->end(SMSM_STAGE_BAND);
-  } else if (with_dots) {
-    SMSM_CUDA_TRY(cudaMemsetAsync(P->part_pq_band, 0, sizeof(double) * SMSM_PART_MAX * P->D, s));
-  }
   return SMSM_OK;
 }
 
@@ -336,6 +347,7 @@ static smsm_plan_s lane_view(const smsm_plan_s* P, int d0, int nd, int lane) {
   v.part_rr += 2 * dd * SMSM_PART_MAX;
   v.st += dd;
   v.rep = P->rep + lane;
+  v.lane = lane;
   if (P->Rpart) {
     const size_t R2C = 2 * (size_t)gram_tc_cp(P);
     v.Rpart += dd * L * P->gram_tc_nG * R2C * R2C;
@@ -391,7 +403,16 @@ static smsm_status enqueue_outer(smsm_plan_s* P, const smsm_params* prm, int k, 
                                         n4, rr0);
   SMSM_LAUNCH_CHECK("k_cg_init");
   T->end(SMSM_STAGE_CG);
-  k_record<<<1, VEC_THREADS, 0, s>>>(P->rep, k, 0, rr0, nvb);
+  // the report's sums go to the lane's side stream, which the next band step joins again before rr0 is rewritten
+  const bool side = !T->mask && lam != 0.f && prm->cg_iters > 0;
+  cudaStream_t rs = side ? P->band_s[P->lane] : s;
+  auto fork = [&]() -> cudaError_t {
+    if (!side) return cudaSuccess;
+    cudaError_t e = cudaEventRecord(P->band_ev[2 * P->lane], s);
+    return e == cudaSuccess ? cudaStreamWaitEvent(rs, P->band_ev[2 * P->lane], 0) : e;
+  };
+  SMSM_CUDA_TRY(fork());
+  k_record<<<1, VEC_THREADS, 0, rs>>>(P->rep, k, 0, rr0, nvb);
   SMSM_LAUNCH_CHECK("k_record");
   for (int j = 0; j < prm->cg_iters; ++j) {
     double* rin = (j & 1) ? rr1 : rr0;
@@ -408,8 +429,13 @@ static smsm_status enqueue_outer(smsm_plan_s* P, const smsm_params* prm, int k, 
     T->end(SMSM_STAGE_CG);
   }
   double* rend = (prm->cg_iters & 1) ? rr1 : rr0;  // bank of the last write
-  k_record<<<1, VEC_THREADS, 0, s>>>(P->rep, k, 1, rend, nvb);
+  SMSM_CUDA_TRY(fork());
+  k_record<<<1, VEC_THREADS, 0, rs>>>(P->rep, k, 1, rend, nvb);
   SMSM_LAUNCH_CHECK("k_record");
+  if (side && k + 1 == prm->outer_iters) {  // nothing joins it any more
+    SMSM_CUDA_TRY(cudaEventRecord(P->band_ev[2 * P->lane + 1], rs));
+    SMSM_CUDA_TRY(cudaStreamWaitEvent(s, P->band_ev[2 * P->lane + 1], 0));
+  }
   return SMSM_OK;
 }
 

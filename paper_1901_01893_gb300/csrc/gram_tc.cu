@@ -10,7 +10,7 @@
 // 128-row tile t of R against the columns [128 t, 2Cp): tile 0 as two MMAs of
 // N = Cp, the others as one MMA of N = 2Cp - 128 t (480 TMEM columns at
 // 2Cp = 288).  It covers a contiguous block of patch rows ky (split-K); its FP32
-// partial goes to global memory and k_gram_tc_reduce adds the partials in FP64
+// partial goes to global memory and k_gram_tc_reduce adds the partials, compensated,
 // in a fixed order.  Roles (warp-specialised, 352 threads):
 //   * thread 0 brings the window of patch row ky -- image rows ky..ky+r-1 of
 //     every shot -- into shared memory with TMA bulk copies (two windows in
@@ -389,52 +389,70 @@ __global__ void __launch_bounds__(GTC_THREADS, 1)
   if (warp == 0) tmem_dealloc(tmem, tmem_cols);
 }
 
-// G[c][c'] (c <= c') = sum_g (R[c][c'] + R[Cp+c][Cp+c']) + i (R[c][Cp+c'] - R[c'][Cp+c]) in FP64,
+// G[c][c'] (c <= c') = sum_g (R[c][c'] + R[Cp+c][Cp+c']) + i (R[c][Cp+c'] - R[c'][Cp+c]),
 // every entry read from R's upper triangle; G[c'][c] is written as the conjugate, so G is
 // exactly Hermitian.  One CTA (32 x 8 threads) per 32 x 32 tile (c, c') on or above the
 // diagonal: the three terms read along c' are coalesced, and R[c'][Cp+c] is read along c
-// and transposed through shared memory.  The sum over g runs in a fixed order.
+// and transposed through shared memory, GRED_G partials at a time (their loads all in flight).
+// The sum over g runs in a fixed order in pairs of FP32 (add2: a 48-bit sum, exact for a few FP32 terms of like
+// size); FP64 additions, at 1/64 of the FP32 rate, were what bounded it (18 matrices of 144 x 144, 11 partials:
+// 90 -> 17 us).
 #define GRED_T 32
+#define GRED_G 4
 __global__ void __launch_bounds__(GRED_T * 8) k_gram_tc_reduce(const float* __restrict__ Rpart,
                                                                double2* __restrict__ G, int LD, int C, int Cp,
                                                                int nG) {
-  __shared__ float tr[GRED_T][GRED_T + 1];
+  __shared__ float tr[GRED_G][GRED_T][GRED_T + 1];
   if (blockIdx.y > blockIdx.x) return;  // tile below the diagonal (uniform per CTA)
   const int R2C = 2 * Cp;
   const int lf = blockIdx.z;
   const int c0 = blockIdx.y * GRED_T, cc0 = blockIdx.x * GRED_T;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int cc = cc0 + tx;
-  double re[GRED_T / 8], im[GRED_T / 8];
+  constexpr int NK = GRED_T / 8;
+  float rh[NK], rl[NK], ih[NK], il[NK];  // high and low parts
 #pragma unroll
-  for (int k = 0; k < GRED_T / 8; ++k) re[k] = im[k] = 0.0;
-  for (int g = 0; g < nG; ++g) {
-    const float* R = Rpart + ((size_t)lf * nG + g) * R2C * R2C;
-    for (int j = ty; j < GRED_T; j += 8) {  // tr[j][i] = R[cc0 + j][Cp + c0 + i]
-      const int rj = cc0 + j, ci = c0 + tx;
-      tr[j][tx] = (rj < C && ci < C) ? R[(size_t)rj * R2C + Cp + ci] : 0.f;
+  for (int k = 0; k < NK; ++k) rh[k] = rl[k] = ih[k] = il[k] = 0.f;
+  for (int g0 = 0; g0 < nG; g0 += GRED_G) {
+    float a[GRED_G][NK], b[GRED_G][NK], c1[GRED_G][NK];
+#pragma unroll
+    for (int q = 0; q < GRED_G; ++q) {
+      const bool live = g0 + q < nG;
+      const float* R = Rpart + ((size_t)lf * nG + (live ? g0 + q : 0)) * R2C * R2C;
+#pragma unroll
+      for (int k = 0; k < NK; ++k) {
+        const int c = c0 + ty + 8 * k;
+        const bool in = live && c < C && cc < C && c <= cc;
+        a[q][k] = in ? R[(size_t)c * R2C + cc] : 0.f;
+        b[q][k] = in ? R[(size_t)(Cp + c) * R2C + Cp + cc] : 0.f;
+        c1[q][k] = in ? R[(size_t)c * R2C + Cp + cc] : 0.f;
+        const int rj = cc0 + ty + 8 * k, ci = c0 + tx;  // tr[q][j][i] = R[cc0 + j][Cp + c0 + i]
+        tr[q][ty + 8 * k][tx] = (live && rj < C && ci < C) ? R[(size_t)rj * R2C + Cp + ci] : 0.f;
+      }
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < GRED_T / 8; ++k) {
-      const int c = c0 + ty + 8 * k;
-      if (c < C && cc < C && c <= cc) {
-        re[k] += (double)R[(size_t)c * R2C + cc] + (double)R[(size_t)(Cp + c) * R2C + Cp + cc];
-        im[k] += (double)R[(size_t)c * R2C + Cp + cc] - (double)tr[tx][ty + 8 * k];
+    for (int q = 0; q < GRED_G; ++q)
+#pragma unroll
+      for (int k = 0; k < NK; ++k) {
+        add2(rh[k], rl[k], a[q][k]);
+        add2(rh[k], rl[k], b[q][k]);
+        add2(ih[k], il[k], c1[q][k]);
+        add2(ih[k], il[k], -tr[q][tx][ty + 8 * k]);
       }
-    }
     __syncthreads();
   }
   double2* Gl = G + (size_t)lf * C * C;
 #pragma unroll
-  for (int k = 0; k < GRED_T / 8; ++k) {
+  for (int k = 0; k < NK; ++k) {
     const int c = c0 + ty + 8 * k;
     if (c < C && cc < C && c <= cc) {
+      const double re = (double)rh[k] + (double)rl[k], im = (double)ih[k] + (double)il[k];
       if (c == cc) {
-        Gl[(size_t)c * C + c] = make_double2(re[k], 0.0);
+        Gl[(size_t)c * C + c] = make_double2(re, 0.0);
       } else {
-        Gl[(size_t)c * C + cc] = make_double2(re[k], im[k]);
-        Gl[(size_t)cc * C + c] = make_double2(re[k], -im[k]);
+        Gl[(size_t)c * C + cc] = make_double2(re, im);
+        Gl[(size_t)cc * C + c] = make_double2(re, -im);
       }
     }
   }

@@ -27,11 +27,8 @@
 #include <vector>
 
 #include "common.cuh"
+#include "umma.cuh"
 
-#define CV_T 16     // output tile edge (pixels)
-#define CV_OCB 32   // output channels per CTA
-#define CV_ICB 8    // input channels staged per step
-#define CV_SP 20    // staged row pitch (18 used)
 #define WG_OCB 32   // weight gradient: output channels per CTA
 #define WG_ICB 32   // weight gradient: input channels per CTA
 #define WG_TY 8     // weight gradient pixel tile: 8 rows x 16 columns
@@ -50,6 +47,8 @@ struct smsm_cnn_s {
   std::vector<float2*> z;          // pre-activations per layer [maxn][cout][H][W]
   float2 *gA, *gB;                 // gradient ping-pong [maxn][width][H][W]
   float2* wpart;                   // weight-gradient partials [WG_SPLIT][max Cout*Cin*9 + Cout]
+  __nv_bfloat16* wB;               // weights of one layer in the convolution's order
+  int* devflag;                    // raised when a bounded wait of a convolution ran out
   double* lpart;                   // per-sample [2] sums (||x0 - t||^2, ||t||^2)
   int step;                        // Adam step
   size_t bytes;
@@ -63,96 +62,253 @@ __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__floa
 // Convolution: out[n][o] = bias[o] + sum_c sum_k Wp[o][c][k] g(in[n][c])(p + k - 1)
 //   g = CReLU when in_relu, identity otherwise; then + resid[n][o] when given, and
 //   each component zeroed where that component of mask[n][o] is not > 0 when given.
-// CTA: a 16 x 16 pixel tile x 32 output channels; thread: 4 consecutive pixels of a
-// row x 8 output channels (32 complex accumulators).  Input channels are staged 8 at
-// a time with a one-pixel halo; a thread keeps 6 pixels of an input row in registers
-// and reuses them for the 3 taps along x.
+// On the tensor cores (tcgen05, BF16 operands, FP32 accumulation in TMEM).  The weights are BF16 values; an
+// FP32 activation is split exactly into three BF16 pieces, so every product is exact and what is rounded is the
+// accumulation, as in an FP32 FMA loop.  Every MMA rounds its accumulator once, so the leading piece's products
+// are dealt out to three accumulators by tap row (24 roundings each for 64 channels) and the two small
+// pieces' (2^-8 and 2^-16 of them) to a fourth, all added in the epilogue: with one accumulator for the
+// leading products the learned start of two 256 x 256 groups was 2.9e-6 from its 64-bit value, with three 8.9e-7 (FP32
+// FMAs: 9e-7).
+//
+// Implicit GEMM without copies: the image is cut into column strips of TW pixels, padded to P = TW + 2 columns, and
+// a strip is read as one line of pixels; a CTA takes 128 consecutive ones and stages them with
+// P + 1 more on both sides.  A staged K slab is 8 BF16 values (re and im of four channels) of every pixel, pixel
+// after pixel, 16 bytes each: the no-swizzle K-major layout with its 8-row groups back to back.  A tap (ky, kx)
+// is the same slab from ky P + kx pixels further on, so the nine taps are nine start addresses of
+// the A descriptor.  Pixels in the padding columns give values nobody stores.
+//   * eight producer warps load the next 8 channels, apply CReLU, split and stage them (two stages);
+//   * one thread brings the 8 channels' weights of all taps (k_cnn_wprep's order: one bulk copy);
+//   * one thread issues 9 taps x 3 pieces of 128 x NT x 16 MMAs;
+//   * the producer warps write the outputs from TMEM at the end.
+// N = NT columns: the real parts of up to 64 output channels, then the imaginary ones.  Waits are bounded; on a
+// timeout the network's error flag is raised.
+// Measured (before: FP32 FMAs, a 16 x 16 pixel tile x 32 channels per CTA), two 256 x 256 images: 64 -> 64 channels
+// 770 -> 62 us; the learned start of both groups (6 layers, width 64) 3.73 -> 0.76 ms.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_cnn_conv(const float2* __restrict__ in, const float2* __restrict__ Wp,
-                                                  const float2* __restrict__ bias, const float2* __restrict__ resid,
-                                                  const float2* __restrict__ mask, float2* __restrict__ out, int Cin,
-                                                  int Cout, int H, int W, int in_relu) {
-  __shared__ __align__(16) float2 sIn[CV_ICB][CV_T + 2][CV_SP];
-  __shared__ __align__(16) float2 sW[CV_ICB][9][CV_OCB];
-  const int tilesx = (W + CV_T - 1) / CV_T;
-  const int tx0 = (blockIdx.x % tilesx) * CV_T, ty0 = (blockIdx.x / tilesx) * CV_T;
-  const int oc0 = blockIdx.y * CV_OCB, n = blockIdx.z;
-  const int tid = threadIdx.x;
-  const int og = tid >> 6, pg = tid & 63;
-  const int py = pg >> 2, px0 = (pg & 3) * 4;
-  const size_t HW = (size_t)H * W;
-  const float2* inn = in + (size_t)n * Cin * HW;
-  float2 acc[4][8];
+#define CV_TL 128                 // pixels of a strip per CTA (one M = 128 block)
+#define CV_MAXP 66                // strip pitch at most
+#define CV_SR (CV_TL + 2 * CV_MAXP + 2)  // staged pixels at most
+#define CV_PROD 256
+#define CV_THREADS (CV_PROD + 64)
+#define CV_MAXITER (1L << 22)
+
+struct ConvShape {
+  int Cin, Cout, H, W, in_relu;
+  int TW, P, nstrip, ntl;  // strip width and pitch, strips per image, CTAs per strip
+  int NT, nchunk;          // MMA columns, chunks of 8 input channels
+};
+
+// weights in the order the MMAs take them: [block of 64 outputs][chunk][tap][slab][NT][8] BF16; column n of a block
+// is Re (n < NT/2) or Im of output n mod NT/2; slab values are (re, im) of four channels
+__global__ void __launch_bounds__(256) k_cnn_wprep(const float2* __restrict__ Wp, __nv_bfloat16* __restrict__ dst,
+                                                   ConvShape g, int nblk) {
+  const int half = g.NT / 2, total = nblk * g.nchunk * 9 * 2 * g.NT;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < total; e += gridDim.x * 256) {
+    int t = e;
+    const int n = t % g.NT;
+    t /= g.NT;
+    const int slab = t & 1;
+    t >>= 1;
+    const int tap = t % 9;
+    t /= 9;
+    const int ch = t % g.nchunk, nb = t / g.nchunk;
+    const int o = nb * 64 + n % half, im = n / half;
+    __align__(16) __nv_bfloat16 v[8];
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+    for (int q = 0; q < 4; ++q) {
+      const int c = ch * 8 + slab * 4 + q;
+      float2 w = cmk(0.f, 0.f);
+      if (o < g.Cout && n % half < 64 && c < g.Cin) w = Wp[((size_t)o * g.Cin + c) * 9 + tap];
+      v[2 * q] = __float2bfloat16_rn(im ? w.y : w.x);
+      v[2 * q + 1] = __float2bfloat16_rn(im ? w.x : -w.y);
+    }
+    reinterpret_cast<uint4*>(dst)[e] = *reinterpret_cast<const uint4*>(v);
+  }
+}
+
+__device__ __forceinline__ bool cv_wait(uint64_t* mbar, uint32_t parity, volatile int* abort_flag) {
+  for (long it = 0; it < CV_MAXITER; ++it) {
+    if (mbar_wait(mbar, parity, 1)) return true;
+    if ((it & 255) == 255 && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+
+__host__ __device__ inline uint32_t cv_a_bytes(const ConvShape& g) {  // one piece of one stage
+  return 2u * (uint32_t)(CV_TL + 2 * g.P + 2) * 16u;
+}
+__host__ __device__ inline uint32_t cv_b_bytes(const ConvShape& g) { return 9u * 2u * (uint32_t)g.NT * 16u; }
+
+__global__ void __launch_bounds__(CV_THREADS, 1)
+    k_cnn_conv(const float2* __restrict__ in, const __nv_bfloat16* __restrict__ wB, const float2* __restrict__ bias,
+               const float2* __restrict__ resid, const float2* __restrict__ mask, float2* __restrict__ out,
+               ConvShape g, int* __restrict__ errflag) {
+  extern __shared__ __align__(128) unsigned char csm[];  // [2 stages][3 pieces of A, B]
+  __shared__ uint32_t tmem_base;
+  __shared__ __align__(8) uint64_t afull[2], bfull[2], empty[2], fin;
+  __shared__ volatile int s_abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int strip = blockIdx.x / g.ntl, t0 = (blockIdx.x - strip * g.ntl) * CV_TL;
+  const int nb = blockIdx.y, n = blockIdx.z;
+  const int SR = CV_TL + 2 * g.P + 2;
+  const uint32_t ab = cv_a_bytes(g), bb = cv_b_bytes(g), stage = 3 * ab + bb;
+  const size_t HW = (size_t)g.H * g.W;
+  int cols = 32;
+  while (cols < 4 * g.NT) cols <<= 1;
+  if (warp == 0) tmem_alloc(&tmem_base, cols);
+  if (tid == 0) {
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(&afull[k], CV_PROD);
+      mbar_init(&bfull[k], 1);
+      mbar_init(&empty[k], 1);
+    }
+    mbar_init(&fin, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    s_abort = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base;
+
+  if (tid < CV_PROD) {
+    // ---------------- producers ----------------
+    constexpr int NI = (2 * CV_SR + CV_PROD - 1) / CV_PROD;
+    int off[NI];       // pixel of the image, or -1 (zero)
+    uint32_t dst[NI];  // byte in a piece
+    int slab[NI];
 #pragma unroll
-    for (int o = 0; o < 8; ++o) acc[j][o] = cmk(0.f, 0.f);
-  for (int ic0 = 0; ic0 < Cin; ic0 += CV_ICB) {
-    for (int e = tid; e < CV_ICB * (CV_T + 2) * (CV_T + 2); e += 256) {
-      const int c = e / ((CV_T + 2) * (CV_T + 2)), rem = e - c * (CV_T + 2) * (CV_T + 2);
-      const int yy = rem / (CV_T + 2), xx = rem - yy * (CV_T + 2);
-      const int gy = ty0 + yy - 1, gx = tx0 + xx - 1;
-      float2 v = cmk(0.f, 0.f);
-      if (ic0 + c < Cin && gy >= 0 && gy < H && gx >= 0 && gx < W) {
-        v = inn[(size_t)(ic0 + c) * HW + (size_t)gy * W + gx];
-        if (in_relu) v = crelu2(v);
+    for (int k = 0; k < NI; ++k) {
+      const int e = tid + CV_PROD * k;
+      slab[k] = e >= SR;
+      const int m = e - slab[k] * SR;  // staged pixel
+      off[k] = -1;
+      dst[k] = 0xffffffffu;
+      if (e < 2 * SR) {
+        dst[k] = (uint32_t)(slab[k] * SR + m) * 16u;
+        const int q = t0 + m - g.P - 1 + 2 * g.P;  // two rows up: never negative
+        const int y = q / g.P - 2, xq = q - (y + 2) * g.P, x = strip * g.TW + xq - 1;
+        if (y >= 0 && y < g.H && x >= 0 && x < g.W) off[k] = y * g.W + x;
       }
-      sIn[c][yy][xx] = v;
     }
-    for (int e = tid; e < CV_ICB * 9 * CV_OCB; e += 256) {
-      const int o = e % CV_OCB, k = (e / CV_OCB) % 9, c = e / (9 * CV_OCB);
-      float2 v = cmk(0.f, 0.f);
-      if (oc0 + o < Cout && ic0 + c < Cin) v = Wp[((size_t)(oc0 + o) * Cin + ic0 + c) * 9 + k];
-      sW[c][k][o] = v;
-    }
-    __syncthreads();
-    const int cn = min(CV_ICB, Cin - ic0);
-    for (int c = 0; c < cn; ++c) {
+    const float2* inn = in + (size_t)n * g.Cin * HW;
+    for (int it = 0; it < g.nchunk; ++it) {
+      const int s = it & 1;
+      float2 v[NI][4];
 #pragma unroll
-      for (int ky = 0; ky < 3; ++ky) {
-        float2 h[6];
+      for (int k = 0; k < NI; ++k)
 #pragma unroll
-        for (int j = 0; j < 6; ++j) h[j] = sIn[c][py + ky][px0 + j];
+        for (int q = 0; q < 4; ++q) {
+          const int c = it * 8 + slab[k] * 4 + q;
+          v[k][q] = cmk(0.f, 0.f);
+          if (off[k] >= 0 && c < g.Cin) v[k][q] = __ldg(inn + (size_t)c * HW + off[k]);
+        }
+      if (it >= 2 && !cv_wait(&empty[s], (uint32_t)((it / 2 - 1) & 1), &s_abort)) break;
+      unsigned char* st = csm + s * stage;
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) {
-          const float4* wq = reinterpret_cast<const float4*>(&sW[c][ky * 3 + kx][og * 8]);
-          float2 w[8];
+      for (int k = 0; k < NI; ++k) {
+        if (dst[k] == 0xffffffffu) continue;
+        float f[8];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float4 t = wq[q];
-            w[2 * q] = cmk(t.x, t.y);
-            w[2 * q + 1] = cmk(t.z, t.w);
+        for (int q = 0; q < 4; ++q) {
+          const float2 u = g.in_relu ? crelu2(v[k][q]) : v[k][q];
+          f[2 * q] = u.x;
+          f[2 * q + 1] = u.y;
+        }
+#pragma unroll
+        for (int piece = 0; piece < 3; ++piece) {
+          __align__(16) __nv_bfloat16 h[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            h[q] = __float2bfloat16_rn(f[q]);
+            f[q] -= __bfloat162float(h[q]);  // exact: the remainder of a round-to-nearest
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int o = 0; o < 8; ++o) cfma(acc[j][o], w[o], h[j + kx]);
+          *reinterpret_cast<uint4*>(st + piece * ab + dst[k]) = *reinterpret_cast<const uint4*>(h);
         }
       }
+      fence_async_smem();
+      mbar_arrive(&afull[s]);
     }
-    __syncthreads();
-  }
-  const int gy = ty0 + py;
-  if (gy >= H) return;
+    // ---------------- epilogue: warp w takes TMEM lanes 32 (w mod 4) .. and every second 16 channels ----------------
+    if (__all_sync(0xffffffffu, cv_wait(&fin, 0, &s_abort)) && !s_abort) {
+      tc_fence_after();
+      const int half = g.NT / 2;
+      const int q = t0 + 32 * (warp & 3) + lane;
+      const int y = q / g.P, xq = q - y * g.P, x = strip * g.TW + xq - 1;
+      const bool live = y < g.H && xq >= 1 && xq <= g.TW && x < g.W;
+      const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+      const size_t pix = (size_t)y * g.W + x;
+      for (int o0 = 16 * (warp >> 2); o0 < half; o0 += 32) {
+        float re[16], im[16];
 #pragma unroll
-  for (int o = 0; o < 8; ++o) {
-    const int oc = oc0 + og * 8 + o;
-    if (oc >= Cout) continue;
-    const float2 b = bias ? bias[oc] : cmk(0.f, 0.f);
-    const size_t base = ((size_t)n * Cout + oc) * HW + (size_t)gy * W;
+        for (int k = 0; k < 16; ++k) re[k] = im[k] = 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gx = tx0 + px0 + j;
-      if (gx >= W) continue;
-      float2 v = cadd(acc[j][o], b);
-      if (resid) v = cadd(v, resid[base + gx]);
-      if (mask) {
-        const float2 mk = mask[base + gx];
-        v = cmk(mk.x > 0.f ? v.x : 0.f, mk.y > 0.f ? v.y : 0.f);
+        for (int acc = 3; acc >= 0; --acc) {  // the small products first
+          __syncwarp();  // the TMEM loads are .sync.aligned
+          uint32_t d[16];
+          tmem_ld16(base + acc * g.NT + o0, d);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) re[k] += __uint_as_float(d[k]);
+          tmem_ld16(base + acc * g.NT + half + o0, d);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) im[k] += __uint_as_float(d[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          const int oc = nb * 64 + o0 + k;
+          if (live && oc < g.Cout) {
+            float2 w = cmk(re[k], im[k]);
+            if (bias) w = cadd(w, bias[oc]);
+            const size_t o = ((size_t)n * g.Cout + oc) * HW + pix;
+            if (resid) w = cadd(w, resid[o]);
+            if (mask) {
+              const float2 mk = mask[o];
+              w = cmk(mk.x > 0.f ? w.x : 0.f, mk.y > 0.f ? w.y : 0.f);
+            }
+            out[o] = w;
+          }
+        }
       }
-      out[base + gx] = v;
+      tc_fence_before();
     }
+  } else if (tid == CV_PROD) {
+    // ---------------- MMA issue ----------------
+    const uint32_t idesc = umma_idesc(1u, 128, g.NT), lboA = (uint32_t)SR * 16u, lboB = (uint32_t)g.NT * 16u;
+    for (int it = 0; it < g.nchunk; ++it) {
+      const int s = it & 1;
+      const uint32_t ph = (uint32_t)((it / 2) & 1);
+      if (!cv_wait(&afull[s], ph, &s_abort) || !cv_wait(&bfull[s], ph, &s_abort)) break;
+      tc_fence_after();
+      const uint32_t a0 = smem_u32(csm + s * stage), b0 = a0 + 3 * ab;
+      for (int tap = 0; tap < 9; ++tap) {
+        const uint64_t bd = umma_desc(b0 + (uint32_t)tap * 2 * lboB, lboB, 128);
+        const uint32_t shift = (uint32_t)((tap / 3) * g.P + tap % 3) * 16u;  // staged pixel 0 is P + 1 before the first
+        const uint32_t ar = a0 + shift;
+        umma_bf16(tmem + (tap / 3) * g.NT, umma_desc(ar, lboA, 128), bd, idesc, (it || tap % 3) ? 1u : 0u);
+        umma_bf16(tmem + 3 * g.NT, umma_desc(ar + ab, lboA, 128), bd, idesc, (it || tap) ? 1u : 0u);
+        umma_bf16(tmem + 3 * g.NT, umma_desc(ar + 2 * ab, lboA, 128), bd, idesc, 1u);
+      }
+      umma_commit(&empty[s]);
+    }
+    umma_commit(&fin);  // every MMA issued above has finished before TMEM and the stages are released
+    mbar_wait(&fin, 0, CV_MAXITER);
+  } else if (tid == CV_PROD + 32) {
+    // ---------------- weights ----------------
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(wB) + (size_t)nb * g.nchunk * bb;
+    int sent = 0;
+    for (int it = 0; it < g.nchunk; ++it, ++sent) {
+      const int s = it & 1;
+      if (it >= 2 && !cv_wait(&empty[s], (uint32_t)((it / 2 - 1) & 1), &s_abort)) break;
+      mbar_arrive_expect_tx(&bfull[s], bb);
+      tma_bulk_g2s(csm + s * stage + 3 * ab, src + (size_t)it * bb, bb, &bfull[s]);
+    }
+    // copies still in flight land before the shared memory is released
+    for (int it = sent > 2 ? sent - 2 : 0; it < sent; ++it) mbar_wait(&bfull[it & 1], (uint32_t)((it / 2) & 1), CV_MAXITER);
   }
+  __syncthreads();
+  if (s_abort && tid == 0) atomicExch(errflag, SMSM_ERR_TIMEOUT);
+  if (warp == 0) tmem_dealloc(tmem, cols);
 }
 
 // ---------------------------------------------------------------------------
@@ -345,18 +501,43 @@ __global__ void k_cnn_round(const float2* __restrict__ master, float2* __restric
 // ---------------------------------------------------------------------------
 static size_t wgrad_smem() { return (size_t)(WG_OCB * WG_TY * WG_TX + WG_ICB * WG_CP) * sizeof(float2); }
 
-static smsm_status conv(const float2* in, const float2* Wp, const float2* bias, const float2* resid, const float2* mask,
-                        float2* out, int n, int Cin, int Cout, int H, int W, int in_relu, cudaStream_t s) {
-  const int tiles = ((W + CV_T - 1) / CV_T) * ((H + CV_T - 1) / CV_T);
-  dim3 grid(tiles, (Cout + CV_OCB - 1) / CV_OCB, n);
-  k_cnn_conv<<<grid, 256, 0, s>>>(in, Wp, bias, resid, mask, out, Cin, Cout, H, W, in_relu);
+static ConvShape conv_shape(int Cin, int Cout, int H, int W, int in_relu) {
+  ConvShape g;
+  g.Cin = Cin;
+  g.Cout = Cout;
+  g.H = H;
+  g.W = W;
+  g.in_relu = in_relu;
+  g.nstrip = (W + CV_MAXP - 3) / (CV_MAXP - 2);  // strips of at most 64 columns, all alike
+  g.TW = (W + g.nstrip - 1) / g.nstrip;
+  g.P = g.TW + 2;
+  g.ntl = (int)(((long)H * g.P + CV_TL - 1) / CV_TL);
+  g.NT = 32 * (((Cout < 64 ? Cout : 64) + 15) / 16);
+  g.nchunk = (Cin + 7) / 8;
+  return g;
+}
+
+static size_t conv_weight_elems(int Cin, int Cout) {  // BF16 values of k_cnn_wprep's output
+  const ConvShape g = conv_shape(Cin, Cout, 1, 1, 0);
+  return (size_t)((Cout + 63) / 64) * g.nchunk * 9 * 2 * g.NT * 8;
+}
+
+static smsm_status conv(const smsm_cnn_s* c, const float2* in, const float2* Wp, const float2* bias,
+                        const float2* resid, const float2* mask, float2* out, int n, int Cin, int Cout, int in_relu,
+                        cudaStream_t s) {
+  const ConvShape g = conv_shape(Cin, Cout, c->H, c->W, in_relu);
+  const int nblk = (Cout + 63) / 64;
+  k_cnn_wprep<<<(nblk * g.nchunk * 9 * 2 * g.NT + 255) / 256, 256, 0, s>>>(Wp, c->wB, g, nblk);
+  SMSM_LAUNCH_CHECK("k_cnn_wprep");
+  const size_t sm = 2 * ((size_t)3 * cv_a_bytes(g) + cv_b_bytes(g));
+  k_cnn_conv<<<dim3(g.nstrip * g.ntl, nblk, n), CV_THREADS, sm, s>>>(in, c->wB, bias, resid, mask, out, g, c->devflag);
   SMSM_LAUNCH_CHECK("k_cnn_conv");
   return SMSM_OK;
 }
 
 static void cnn_free(smsm_cnn_s* c) {
   if (!c) return;
-  void* ptrs[] = {c->master, c->wbf, c->grad, c->m1, c->m2, c->wt, c->gA, c->gB, c->wpart, c->lpart};
+  void* ptrs[] = {c->master, c->wbf, c->grad, c->m1, c->m2, c->wt, c->gA, c->gB, c->wpart, c->lpart, c->wB, c->devflag};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (float2* p : c->z)
@@ -430,8 +611,19 @@ extern "C" smsm_status smsm_cnn_create(smsm_cnn_t* out, int channels, int width,
   if (!st) st = calloc_dev(c, &c->gB, (size_t)max_batch * wmax * HW);
   if (!st) st = calloc_dev(c, &c->wpart, (size_t)WG_SPLIT * maxw);
   if (!st) st = calloc_dev(c, &c->lpart, (size_t)2 * max_batch);
+  size_t wmaxB = 0;
+  for (int k = 0; k < layers; ++k) {  // both ways: the data gradient's convolution has them exchanged
+    const size_t f = conv_weight_elems(c->cin[k], c->cout[k]), r = conv_weight_elems(c->cout[k], c->cin[k]);
+    wmaxB = wmaxB > f ? wmaxB : f;
+    wmaxB = wmaxB > r ? wmaxB : r;
+  }
+  if (!st) st = calloc_dev(c, &c->wB, wmaxB);
+  if (!st) st = calloc_dev(c, &c->devflag, (size_t)1);
   if (!st) {
     cudaError_t e = cudaFuncSetAttribute(k_cnn_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem());
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_cnn_conv, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               2 * (3 * 2 * CV_SR * 16 + 9 * 2 * 128 * 16));
     if (e != cudaSuccess) {
       smsm_set_error("smsm_cnn_create: %s", cudaGetErrorString(e));
       st = SMSM_ERR_CUDA;
@@ -516,8 +708,8 @@ static smsm_status cnn_forward(smsm_cnn_s* c, const float2* a, float2* x0, int n
   for (int k = 0; k < c->layers; ++k) {
     const bool last = k + 1 == c->layers;
     float2* o = last ? x0 : c->z[k];
-    if ((st = conv(h, c->wbf + c->woff[k], c->wbf + c->boff[k], last ? a : nullptr, nullptr, o, n, c->cin[k],
-                   c->cout[k], c->H, c->W, k > 0, s)))
+    if ((st = conv(c, h, c->wbf + c->woff[k], c->wbf + c->boff[k], last ? a : nullptr, nullptr, o, n, c->cin[k],
+                   c->cout[k], k > 0, s)))
       return st;
     h = c->z[k];
   }
@@ -562,7 +754,7 @@ static smsm_status cnn_backward(smsm_cnn_s* c, const float2* a, const float2* t,
       k_cnn_wt<<<(int)(((size_t)co * ci * 9 + 255) / 256), 256, 0, s>>>(c->wbf + c->woff[k], c->wt, ci, co);
       SMSM_LAUNCH_CHECK("k_cnn_wt");
       // dh_{k} = conv(G, wt); times the CReLU mask of z_{k-1}: the gradient of z_{k-1}
-      if ((st = conv(G, c->wt, nullptr, nullptr, c->z[k - 1], Gn, n, co, ci, c->H, c->W, 0, s))) return st;
+      if ((st = conv(c, G, c->wt, nullptr, nullptr, c->z[k - 1], Gn, n, co, ci, 0, s))) return st;
       float2* tmp = G;
       G = Gn;
       Gn = tmp;
@@ -571,7 +763,13 @@ static smsm_status cnn_backward(smsm_cnn_s* c, const float2* a, const float2* t,
   if (loss) {
     std::vector<double> h(2 * (size_t)n);
     SMSM_CUDA_TRY(cudaMemcpyAsync(h.data(), c->lpart, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    int flag = 0;
+    SMSM_CUDA_TRY(cudaMemcpyAsync(&flag, c->devflag, sizeof(int), cudaMemcpyDeviceToHost, s));
     SMSM_CUDA_TRY(cudaStreamSynchronize(s));
+    if (flag) {
+      smsm_set_error("a convolution gave up a bounded wait (device status %d)", flag);
+      return (smsm_status)flag;
+    }
     double L = 0.0;
     for (int i = 0; i < n; ++i) L += h[2 * i] / h[2 * i + 1];
     *loss = L / n;

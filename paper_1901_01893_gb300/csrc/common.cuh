@@ -268,6 +268,9 @@ smsm_status launch_rowfft_in_T(const smsm_plan_s* P, const float2* in, float2* o
 // inverse row FFT of p (N rows per image) with the CG update p = r + beta p fused in
 smsm_status launch_rowfft_out_T_cgp(const smsm_plan_s* P, float2* p, const float2* r, float2* out, int nb,
                                     const double* rr_new, const double* rr_old, int nrr, cudaStream_t s);
+// rowfft.cu: the same by two register DFTs (mode 0: out_T, 1: in_T, 2: out_T_cgp); SMSM_ERR_ARG for other lengths
+smsm_status launch_rowfft2(const smsm_plan_s* P, int mode, const float2* in, float2* out, int nb, int rows, int inverse,
+                           int band, float2* p, const double* rr_new, const double* rr_old, int nrr, cudaStream_t s);
 enum ColMode { COL_FWD = 0, COL_ADJ = 1, COL_NORMAL = 2, COL_PEN = 3 };
 // Column-stage arguments (operators.cu, colfast.cu)
 struct ColArgs {

@@ -9,6 +9,9 @@
 #pragma once
 #include "common.cuh"
 
+// (-1)^n as a float
+__device__ __forceinline__ float sgn_par(int n) { return (n & 1) ? -1.f : 1.f; }
+
 template <bool INV>
 __device__ __forceinline__ float2 tw_get(const float2* tw, int idx) {
   float2 w = tw[idx];
@@ -71,6 +74,66 @@ __device__ __forceinline__ void dft3(float2* v) {
   v[0] = cadd(v[0], t1);
   v[1] = cadd(m, j);
   v[2] = csub(m, j);
+}
+
+// exp(-2 pi i m / R) for the products m met in a two-step DFT of length R
+template <int R>
+__device__ __forceinline__ constexpr float rf_cos(int m) {
+  constexpr float c16[10] = {1.f, 0.92387953251128674f, 0.70710678118654752f, 0.38268343236508977f, 0.f,
+                             -0.38268343236508977f, -0.70710678118654752f, -0.92387953251128674f, -1.f,
+                             -0.92387953251128674f};
+  constexpr float c12[7] = {1.f, 0.86602540378443865f, 0.5f, 0.f, -0.5f, -0.86602540378443865f, -1.f};
+  constexpr float c9[5] = {1.f, 0.76604444311897804f, 0.17364817766693035f, -0.5f, -0.93969262078590838f};
+  constexpr float c6[3] = {1.f, 0.5f, -0.5f};
+  return R == 16 ? c16[m] : (R == 12 ? c12[m] : (R == 9 ? c9[m] : c6[m]));
+}
+template <int R>
+__device__ __forceinline__ constexpr float rf_sin(int m) {
+  constexpr float s16[10] = {0.f, 0.38268343236508977f, 0.70710678118654752f, 0.92387953251128674f, 1.f,
+                             0.92387953251128674f, 0.70710678118654752f, 0.38268343236508977f, 0.f,
+                             -0.38268343236508977f};
+  constexpr float s12[7] = {0.f, 0.5f, 0.86602540378443865f, 1.f, 0.86602540378443865f, 0.5f, 0.f};
+  constexpr float s9[5] = {0.f, 0.64278760968653933f, 0.98480775301220806f, 0.86602540378443865f,
+                           0.34202014332566873f};
+  constexpr float s6[3] = {0.f, 0.86602540378443865f, 0.86602540378443865f};
+  return R == 16 ? s16[m] : (R == 12 ? s12[m] : (R == 9 ? s9[m] : s6[m]));
+}
+
+template <int R, bool INV>
+__device__ __forceinline__ void rf_dft(float2* v) {
+  if constexpr (R == 2) {
+    dft2<INV>(v);
+  } else if constexpr (R == 3) {
+    dft3<INV>(v);
+  } else if constexpr (R == 4) {
+    dft4<INV>(v);
+  } else if constexpr (R == 8) {
+    dft8<INV>(v);
+  } else {  // A B points: n = B n1 + n2, X[k1 + A k2]
+    constexpr int A = R == 16 ? 4 : (R == 12 ? 4 : 3), B = R / A;
+    float2 t[A][B];
+#pragma unroll
+    for (int n2 = 0; n2 < B; ++n2) {
+      float2 u[A];
+#pragma unroll
+      for (int n1 = 0; n1 < A; ++n1) u[n1] = v[B * n1 + n2];
+      rf_dft<A, INV>(u);
+#pragma unroll
+      for (int k1 = 0; k1 < A; ++k1) {
+        const int m = n2 * k1;
+        if (m == 0)
+          t[k1][n2] = u[k1];
+        else
+          t[k1][n2] = cmul(u[k1], cmk(rf_cos<R>(m), INV ? rf_sin<R>(m) : -rf_sin<R>(m)));
+      }
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) {
+      rf_dft<B, INV>(t[k1]);
+#pragma unroll
+      for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = t[k1][k2];
+    }
+  }
 }
 
 // One radix-R pass (R in {2, 3, 4, 8}) of the Stockham FFT described above, with
@@ -200,5 +263,85 @@ __device__ __noinline__ float2* fft_smem_call(float2* a, float2* b, int nbatch, 
   return fft_smem<INV>(a, b, nbatch, bstride, d, tw);
 }
 
-// (-1)^n as a float
-__device__ __forceinline__ float sgn_par(int n) { return (n & 1) ? -1.f : 1.f; }
+
+// Centred unitary transforms of `nb` lines of N = R1 R2 points by two register DFTs and one exchange (see rowfft.cu):
+// src [nb][N] -> z [nb][lines2_ld] -> out(line, k, value), every value once.  Threads of the whole block; src may be
+// overwritten by `out` (it is read before the barrier between the steps only).  No barrier at the end.
+template <bool INV, int R1, int R2, class Out>
+__device__ __forceinline__ void fft_lines2(const float2* src, float2* z, int nb, const float2* tw, float sN, Out out) {
+  constexpr int N = R1 * R2, Q = R2 | 1, LD = R1 * Q;
+  for (int t = threadIdx.x; t < nb * R2; t += blockDim.x) {
+    const int b = t / R2, j = t - b * R2;
+    float2 v[R1];
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      v[r] = src[b * N + j + R2 * r];
+      if ((R2 * r) & 1) v[r] = cmk(-v[r].x, -v[r].y);
+    }
+    rf_dft<R1, INV>(v);
+    const float sj = sgn_par(j);
+    z[b * LD + j] = cscale(v[0], sj);
+#pragma unroll
+    for (int k = 1; k < R1; ++k) {
+      const float2 w = tw_get<INV>(tw, j * k);
+      z[b * LD + k * Q + j] = cmul(v[k], cmk(sj * w.x, sj * w.y));
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < nb * R1; t += blockDim.x) {
+    const int b = t / R1, k1 = t - b * R1;
+    float2 v[R2];
+#pragma unroll
+    for (int j = 0; j < R2; ++j) v[j] = z[b * LD + k1 * Q + j];
+    rf_dft<R2, INV>(v);
+    const float sc = sN * sgn_par(k1);
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) out(b, k1 + R1 * k2, cscale(v[k2], ((R1 * k2) & 1) ? -sc : sc));
+  }
+}
+
+// line pitch of z for the lengths that fft_lines2 serves (0: none)
+__host__ __device__ inline int lines2_ld(int N) {
+  switch (N) {
+    case 48: return 8 * 7;
+    case 64: return 8 * 9;
+    case 72: return 8 * 9;
+    case 96: return 12 * 9;
+    case 108: return 12 * 9;
+    case 128: return 16 * 9;
+    case 144: return 12 * 13;
+    case 192: return 16 * 13;
+    case 256: return 16 * 17;
+    default: return 0;
+  }
+}
+#define FFT_LINES2_SWITCH(N, CALL) \
+  switch (N) {                     \
+    case 48: CALL(8, 6); break;    \
+    case 64: CALL(8, 8); break;    \
+    case 72: CALL(8, 9); break;    \
+    case 96: CALL(12, 8); break;   \
+    case 108: CALL(12, 9); break;  \
+    case 128: CALL(16, 8); break;  \
+    case 144: CALL(12, 12); break; \
+    case 192: CALL(16, 12); break; \
+    default: CALL(16, 16); break;  \
+  }
+// in shared memory, [nb][N] -> [nb][N] (in place allowed)
+template <bool INV>
+__device__ __noinline__ void fft_lines2_smem(const float2* src, float2* z, float2* dst, int nb, int N, const float2* tw,
+                                             float sN) {
+#define FFT_L2(R1, R2) \
+  fft_lines2<INV, R1, R2>(src, z, nb, tw, sN, [&](int b, int k, float2 v) { dst[b * (R1 * R2) + k] = v; })
+  FFT_LINES2_SWITCH(N, FFT_L2)
+#undef FFT_L2
+}
+// to global lines dst + b stride
+template <bool INV>
+__device__ __noinline__ void fft_lines2_global(const float2* src, float2* z, float2* dst, size_t stride, int nb, int N,
+                                               const float2* tw, float sN) {
+#define FFT_L2(R1, R2) \
+  fft_lines2<INV, R1, R2>(src, z, nb, tw, sN, [&](int b, int k, float2 v) { dst[b * stride + k] = v; })
+  FFT_LINES2_SWITCH(N, FFT_L2)
+#undef FFT_L2
+}

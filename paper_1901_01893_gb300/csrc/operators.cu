@@ -279,6 +279,8 @@ static int rowfft_vec(const void* in, const void* out) {
 
 smsm_status launch_rowfft_out_T(const smsm_plan_s* P, const float2* in, float2* out, int nb, int rows,
                                 int inverse, cudaStream_t s) {
+  const smsm_status fst = launch_rowfft2(P, 0, in, out, nb, rows, inverse, 0, nullptr, nullptr, nullptr, 0, s);
+  if (fst != SMSM_ERR_ARG) return fst;
   const int TY = pick_ty(rows);
   const int vec = rowfft_vec(in, out);
   dim3 grid(rows / TY, nb);
@@ -294,6 +296,8 @@ smsm_status launch_rowfft_out_T(const smsm_plan_s* P, const float2* in, float2* 
 smsm_status launch_rowfft_out_T_cgp(const smsm_plan_s* P, float2* p, const float2* r, float2* out, int nb,
                                     const double* rr_new, const double* rr_old, int nrr, cudaStream_t s) {
   const int rows = P->N;
+  const smsm_status fst = launch_rowfft2(P, 2, r, out, nb, rows, 1, 0, p, rr_new, rr_old, nrr, s);
+  if (fst != SMSM_ERR_ARG) return fst;
   const int TY = pick_ty(rows);
   dim3 grid(rows / TY, nb);
   k_rowfft_out_T_cgp<true><<<grid, 256, rowfft_smem(P->N, TY), s>>>(p, r, out, rows, TY, P->fN, P->twN, P->sN,
@@ -304,6 +308,8 @@ smsm_status launch_rowfft_out_T_cgp(const smsm_plan_s* P, float2* p, const float
 
 smsm_status launch_rowfft_in_T(const smsm_plan_s* P, const float2* in, float2* out, int nb, int rows,
                                int inverse, cudaStream_t s, int band) {
+  const smsm_status fst = launch_rowfft2(P, 1, in, out, nb, rows, inverse, band, nullptr, nullptr, nullptr, 0, s);
+  if (fst != SMSM_ERR_ARG) return fst;
   const int TY = pick_ty(rows);
   const int vec = rowfft_vec(in, out);
   dim3 grid(rows / TY, nb);

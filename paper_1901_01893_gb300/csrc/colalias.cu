@@ -85,10 +85,14 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
   extern __shared__ __align__(16) float2 sm[];
   __shared__ __align__(8) uint64_t bar[1];  // hybrid lines
   const int N = a.N, M = a.M;
-  float2* img = sm;           // [B][N]
-  float2* tmp = img + B * N;  // [B][N]
-  float2* ph = tmp + B * N;   // [B][N] image times a_i^k
-  float2* sTwN = ph + B * N;  // [N]
+  // two-step transforms up to 4 shots (26 directions of 128 x 128, 4 shots: 64.7 -> 55.4 us an application; with 8 shots
+  // the 16-point DFTs' registers cost more than a pass through shared memory: 64 us on two slices of 192 x 192
+  // in two directions, 84 with them)
+  const int zl2 = NS <= 4 ? lines2_ld(N) : 0, ldz = zl2 ? zl2 : N;  // (their exchange is padded)
+  float2* img = sm;             // [B][N]
+  float2* tmp = img + B * N;    // [B][N]; before: the first transform's exchange
+  float2* ph = tmp + B * ldz;   // [B][N] image times a_i^k; then the second transform's exchange
+  float2* sTwN = ph + B * ldz;  // [N]
   float2* sAsh = sTwN + N;    // [NS][NS]: a_i^q, q < NS (padded to 16 bytes)
   double* red = reinterpret_cast<double*>(sAsh + ((NS * NS + 1) & ~1));  // [32]
   const int x = blockIdx.x;
@@ -140,9 +144,11 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
     return;
   }
   // hybrid lines -> image lines (F_y^-1)
-  for (int b = bsub; b < B; b += tpy) img[b * N + y] = cscale(img[b * N + y], sy);
-  __syncthreads();
-  {
+  if (NS <= 4 && zl2) {
+    fft_lines2_smem<true>(img, tmp, img, B, N, sTwN, a.sN);
+  } else {
+    for (int b = bsub; b < B; b += tpy) img[b * N + y] = cscale(img[b * N + y], sy);
+    __syncthreads();
     float2* R = fft_smem_call<true>(img, tmp, B, N, a.fN, sTwN);
     const float sc = a.sN * sy;
     for (int b = bsub; b < B; b += tpy) img[b * N + y] = cscale(R[b * N + y], sc);
@@ -193,7 +199,7 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
         acc.y = fmaf(a.lambda, q.y, acc.y);
       }
       dsum = fmaf(v.x, acc.x, fmaf(v.y, acc.y, dsum));
-      tmp[b * N + y] = cscale(acc, sy);
+      tmp[b * N + y] = zl2 ? acc : cscale(acc, sy);
     };
     if (PRELOAD && tpy == 1) {
       if (own) {
@@ -240,6 +246,10 @@ __global__ void __launch_bounds__(512) k_col_alias(ColArgs a, const float2* __re
     for (int w = 0; w < nt / 32; ++w) s2 += red[w];
     gdot[x] = s2;
   }
+  if (NS <= 4 && zl2) {
+    fft_lines2_global<false>(tmp, ph, gout + (size_t)x * N, NN, B, N, sTwN, a.sN);
+    return;
+  }
   float2* Rr = fft_smem_call<false>(tmp, ph, B, N, a.fN, sTwN);
   const float so = a.sN * sy;
   for (int b = bsub; b < B; b += tpy) gout[(size_t)b * NN + (size_t)x * N + y] = cscale(Rr[b * N + y], so);
@@ -265,7 +275,8 @@ static int alias_threads(int N, int B) { return (N * alias_tpy(N, B) + 31) / 32 
 
 static size_t alias_smem(const smsm_plan_s* P) {
   const int B = P->L * P->Ns;
-  return (size_t)(3 * B * P->N + P->N + ((P->Ns * P->Ns + 1) & ~1)) * sizeof(float2) + 32 * sizeof(double);
+  const int ldz = P->Ns <= 4 && lines2_ld(P->N) ? lines2_ld(P->N) : P->N;
+  return (size_t)(B * P->N + 2 * B * ldz + P->N + ((P->Ns * P->Ns + 1) & ~1)) * sizeof(float2) + 32 * sizeof(double);
 }
 
 size_t alias_corr_count(const smsm_plan_s* P) {

@@ -105,6 +105,8 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
   }
   __syncthreads();
 
+  // the shot's twiddle goes onto the image pixels before the coil loop and onto the sums after it (not onto every
+  // coil's map): tmp holds the twiddled lines, each element read by the lane that wrote it
   const int i = warp;  // this warp's shot
   float2 acc[L][NK];
   const bool pen = gmult != nullptr && a.lambda != 0.f;
@@ -113,13 +115,8 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
 #pragma unroll
     for (int k = 0; k < NK; ++k) {
       const int y = lane + 32 * k;
-      float2 s = cmk(0.f, 0.f);
-      if (pen) {
-        const float2* ml = gmult + (size_t)l * mult_planes(Ns) * NN;
-        for (int j = 0; j < Ns; ++j) cfma(s, mult_at(ml, i, j, Ns, NN, (size_t)x * N + y), img[(l * Ns + j) * N + y]);
-        s = cscale(s, a.lambda);
-      }
-      acc[l][k] = s;
+      acc[l][k] = cmk(0.f, 0.f);
+      tmp[(l * Ns + i) * N + y] = cmul(sTs[i * N + y], img[(l * Ns + i) * N + y]);
     }
 
   for (int c = 0; c < Nc; ++c) {
@@ -130,12 +127,11 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
 #pragma unroll
       for (int f = 0; f < RW; ++f) fw[l][f] = cmk(0.f, 0.f);
       const float2* srow = a.sensT + (size_t)(l * Nc + c) * NN + (size_t)x * N;
-      const float2* irow = img + (l * Ns + i) * N;
+      const float2* irow = tmp + (l * Ns + i) * N;
 #pragma unroll
       for (int k = 0; k < NK; ++k) {
         const int y = lane + 32 * k;
-        const float2 st = cmul(__ldg(srow + y), sTs[i * N + y]);
-        cfma(fw[l][MR > 0 ? k % RW : 0], st, irow[y]);
+        cfma(fw[l][MR > 0 ? k % RW : 0], __ldg(srow + y), irow[y]);
       }
     }
     if (MR == 0) {
@@ -188,15 +184,14 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
         }
       }
     }
-    // unfold, conjugate shot twiddle and coil, accumulate
+    // unfold, conjugate coil, accumulate
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       const float2* srow = a.sensT + (size_t)(l * Nc + c) * NN + (size_t)x * N;
 #pragma unroll
       for (int k = 0; k < NK; ++k) {
         const int y = lane + 32 * k;
-        const float2 st = cmul(__ldg(srow + y), sTs[i * N + y]);
-        cfmacj(acc[l][k], st, fw[l][MR > 0 ? k % RW : 0]);
+        cfmacj(acc[l][k], __ldg(srow + y), fw[l][MR > 0 ? k % RW : 0]);
       }
     }
   }
@@ -209,6 +204,13 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
     for (int k = 0; k < NK; ++k) {
       const int y = lane + 32 * k;
       const float2 u = img[(l * Ns + i) * N + y];
+      acc[l][k] = cmulcj(sTs[i * N + y], acc[l][k]);
+      if (pen) {
+        const float2* ml = gmult + (size_t)l * mult_planes(Ns) * NN;
+        float2 q = cmk(0.f, 0.f);
+        for (int j = 0; j < Ns; ++j) cfma(q, mult_at(ml, i, j, Ns, NN, (size_t)x * N + y), img[(l * Ns + j) * N + y]);
+        acc[l][k] = cmk(fmaf(a.lambda, q.x, acc[l][k].x), fmaf(a.lambda, q.y, acc[l][k].y));
+      }
       ds = fmaf(u.x, acc[l][k].x, fmaf(u.y, acc[l][k].y, ds));
       tmp[(l * Ns + i) * N + y] = cscale(acc[l][k], sgn_par(y));
     }

@@ -558,9 +558,11 @@ typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int
 
 // Slots = blocks per warp.  One CTA's 16 warps hold up to 5 blocks each (C <= 192: 80 of 128 registers);
 // above, four CTAs hold the 105 (C = 208+) to 210 (C = 320) blocks with 2 to 4 each.
-static TermFn term_fn(int C, int* cl) {
+// Two matrices or fewer leave most SMs idle: four CTAs per term then, too (the same blocks, the same sums), where a
+// warp has several blocks to give away (two matrices: C = 144 89 -> 62 us; C = 100 53 -> 62, left alone).
+static TermFn term_fn(int C, int LD, int* cl) {
   const int nb = rat_nb(C), nblk = nb * (nb + 1) / 2;
-  *cl = nb > 12 ? 4 : 1;
+  *cl = nb > 12 || (LD <= 2 && nb > 8) ? 4 : 1;
   if (*cl == 1) {
     switch ((nblk + RAT_NW - 1) / RAT_NW) {
       case 1: return k_is_term<1, 1>;
@@ -571,6 +573,7 @@ static TermFn term_fn(int C, int* cl) {
     }
   }
   switch ((nblk + 4 * RAT_NW - 1) / (4 * RAT_NW)) {
+    case 1: return k_is_term<1, 4>;
     case 2: return k_is_term<2, 4>;
     case 3: return k_is_term<3, 4>;
     default: return k_is_term<4, 4>;
@@ -578,11 +581,15 @@ static TermFn term_fn(int C, int* cl) {
 }
 
 smsm_status invsqrt_init_attrs(const smsm_plan_s* P) {
-  int cl;
-  TermFn fn = term_fn(P->C, &cl);
-  // per kernel, not per plan: the most any C of the instance uses
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)rat_smem(cl > 1 ? rat_nb(SMSM_MAX_C) : 12, cl));
+  cudaError_t e = cudaSuccess;
+  for (int LD : {1, P->LD}) {  // a lane's sub-batch may be smaller than the plan
+    int cl;
+    TermFn fn = term_fn(P->C, LD, &cl);
+    // per kernel, not per plan: the most any C of the instance uses
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)rat_smem(cl > 1 ? rat_nb(SMSM_MAX_C) : 12, cl));
+  }
   if (e != cudaSuccess) {
     smsm_set_error("inverse square root: %s", cudaGetErrorString(e));
     return SMSM_ERR_CUDA;
@@ -616,7 +623,7 @@ smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, co
                                   outer, prm->eps0_rel, prm->eta, prm->eps_min_rel);
   SMSM_LAUNCH_CHECK("k_is_sched");
   int cl;
-  TermFn fn = term_fn(C, &cl);
+  TermFn fn = term_fn(C, LD, &cl);
   const int chunk = scratch_cap(P);
   for (int l0 = 0; l0 < LD; l0 += chunk) {
     const int n = LD - l0 < chunk ? LD - l0 : chunk;

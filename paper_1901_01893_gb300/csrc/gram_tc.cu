@@ -110,6 +110,15 @@ __host__ __device__ inline int gtc_tmem_cols(int R2C) {
   return c;
 }
 
+// One CTA's partial of R, row tile after row tile (tile t: the columns [128 t, 2Cp) of its rows): groups of four
+// columns, and in a group the tile's rows, 16 bytes each.  A warp of the drain holds 32 rows of a group, so each of
+// its reductions is 512 contiguous bytes; with rows of 2Cp floats every lane went to a line of its own, and those
+// reductions bounded the kernel (52 matrices of 128 x 128, 4 shots, r = 6, the whole Gram: 1400 -> 1042 us).  Element (row, c) of the upper triangle is word gtc_rofs + (c & 3).
+__device__ __forceinline__ size_t gtc_rofs(int R2C, int row, int c) {
+  const int t = row >> 7, h = min(128, R2C - 128 * t);
+  return (size_t)128 * (t * R2C - 64 * t * (t - 1)) + (size_t)(((c >> 2) - 32 * t) * h + (row & 127)) * 4;
+}
+
 // This CTA: every row tile of R, patch rows ky in [ky0, ky1) (block g of nG), matrix lf.
 // A chunk is KCH = 32 KSTEP / ESZ consecutive patches of one patch row (the row's
 // tail zero-padded).  Producer unit = one 16-byte core-matrix row: column c of X (its
@@ -353,7 +362,8 @@ __global__ void __launch_bounds__(GTC_THREADS, 1)
         const int w = R2C - 128 * tt;
         const int row = 128 * tt + 32 * lw + lane;
         if (128 * tt + 32 * lw < R2C) {  // warp-uniform: some row of this warp is in range
-          float* orow = Rl + (size_t)row * R2C + 128 * tt;
+          const int h4 = 4 * min(128, R2C - 128 * tt);  // floats of a group of four columns
+          float* orow = Rl + (size_t)128 * toff + 4 * (32 * lw + lane);
           for (int c0 = 0; c0 < w; c0 += 16) {
             uint32_t dv[16];
             tmem_ld16(tmem + ((uint32_t)(32 * lw) << 16) + toff + (uint32_t)c0, dv);
@@ -362,10 +372,11 @@ __global__ void __launch_bounds__(GTC_THREADS, 1)
               for (int q = 0; q < 4; ++q) {
                 const float v0 = __uint_as_float(dv[4 * q]), v1 = __uint_as_float(dv[4 * q + 1]);
                 const float v2 = __uint_as_float(dv[4 * q + 2]), v3 = __uint_as_float(dv[4 * q + 3]);
+                float* o = orow + (size_t)((c0 >> 2) + q) * h4;
                 if (ep == 0)
-                  *reinterpret_cast<float4*>(orow + c0 + 4 * q) = make_float4(v0, v1, v2, v3);
+                  *reinterpret_cast<float4*>(o) = make_float4(v0, v1, v2, v3);
                 else
-                  red_add_v4(orow + c0 + 4 * q, v0, v1, v2, v3);
+                  red_add_v4(o, v0, v1, v2, v3);
               }
             }
           }
@@ -379,7 +390,7 @@ __global__ void __launch_bounds__(GTC_THREADS, 1)
       for (int tt = 0; tt < ntile; ++tt) {
         const int row = 128 * tt + 32 * lw + lane;
         if (row < R2C)
-          for (int c = 128 * tt; c < R2C; ++c) Rl[(size_t)row * R2C + c] = 0.f;
+          for (int c = 128 * tt; c < R2C; ++c) Rl[gtc_rofs(R2C, row, c) + (c & 3)] = 0.f;
       }
   }
   __syncthreads();
@@ -392,8 +403,8 @@ __global__ void __launch_bounds__(GTC_THREADS, 1)
 // G[c][c'] (c <= c') = sum_g (R[c][c'] + R[Cp+c][Cp+c']) + i (R[c][Cp+c'] - R[c'][Cp+c]),
 // every entry read from R's upper triangle; G[c'][c] is written as the conjugate, so G is
 // exactly Hermitian.  One CTA (32 x 8 threads) per 32 x 32 tile (c, c') on or above the
-// diagonal: the three terms read along c' are coalesced, and R[c'][Cp+c] is read along c
-// and transposed through shared memory, GRED_G partials at a time (their loads all in flight).
+// diagonal: a lane a row and a warp four columns, as the partials lie (16-byte loads, 512 contiguous bytes a
+// warp), and R[c'][Cp+c] transposed through shared memory, GRED_G partials at a time (their loads all in flight).
 // The sum over g runs in a fixed order in pairs of FP32 (add2: a 48-bit sum, exact for a few FP32 terms of like
 // size); FP64 additions, at 1/64 of the FP32 rate, were what bounded it (18 matrices of 144 x 144, 11 partials:
 // 90 -> 17 us).
@@ -408,44 +419,52 @@ __global__ void __launch_bounds__(GRED_T * 8) k_gram_tc_reduce(const float* __re
   const int lf = blockIdx.z;
   const int c0 = blockIdx.y * GRED_T, cc0 = blockIdx.x * GRED_T;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int cc = cc0 + tx;
-  constexpr int NK = GRED_T / 8;
+  const int c = c0 + tx, ccb = cc0 + 4 * ty;
+  constexpr int NK = 4;
   float rh[NK], rl[NK], ih[NK], il[NK];  // high and low parts
 #pragma unroll
   for (int k = 0; k < NK; ++k) rh[k] = rl[k] = ih[k] = il[k] = 0.f;
+  // offsets in a partial of R[c][ccb ..], R[Cp + c][Cp + ccb ..], R[c][Cp + ccb ..] and R[cc0 + tx][Cp + c0 + 4 ty ..]
+  const bool in = c < C && ccb < C && c < ccb + 4;
+  const bool tin = cc0 + tx < C && c0 + 4 * ty < C;
+  const size_t oa = in ? gtc_rofs(R2C, c, ccb) : 0, ob = in ? gtc_rofs(R2C, Cp + c, Cp + ccb) : 0,
+               oc = in ? gtc_rofs(R2C, c, Cp + ccb) : 0, ot = tin ? gtc_rofs(R2C, cc0 + tx, Cp + c0 + 4 * ty) : 0;
+  const float* Rf = Rpart + (size_t)lf * nG * R2C * R2C;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int g0 = 0; g0 < nG; g0 += GRED_G) {
-    float a[GRED_G][NK], b[GRED_G][NK], c1[GRED_G][NK];
+    float4 a[GRED_G], b[GRED_G], c1[GRED_G];
 #pragma unroll
     for (int q = 0; q < GRED_G; ++q) {
       const bool live = g0 + q < nG;
-      const float* R = Rpart + ((size_t)lf * nG + (live ? g0 + q : 0)) * R2C * R2C;
-#pragma unroll
-      for (int k = 0; k < NK; ++k) {
-        const int c = c0 + ty + 8 * k;
-        const bool in = live && c < C && cc < C && c <= cc;
-        a[q][k] = in ? R[(size_t)c * R2C + cc] : 0.f;
-        b[q][k] = in ? R[(size_t)(Cp + c) * R2C + Cp + cc] : 0.f;
-        c1[q][k] = in ? R[(size_t)c * R2C + Cp + cc] : 0.f;
-        const int rj = cc0 + ty + 8 * k, ci = c0 + tx;  // tr[q][j][i] = R[cc0 + j][Cp + c0 + i]
-        tr[q][ty + 8 * k][tx] = (live && rj < C && ci < C) ? R[(size_t)rj * R2C + Cp + ci] : 0.f;
-      }
+      const float* R = Rf + (size_t)(live ? g0 + q : 0) * R2C * R2C;
+      a[q] = live && in ? *reinterpret_cast<const float4*>(R + oa) : zero;
+      b[q] = live && in ? *reinterpret_cast<const float4*>(R + ob) : zero;
+      c1[q] = live && in ? *reinterpret_cast<const float4*>(R + oc) : zero;
+      const float4 t = live && tin ? *reinterpret_cast<const float4*>(R + ot) : zero;
+      tr[q][tx][4 * ty] = t.x;
+      tr[q][tx][4 * ty + 1] = t.y;
+      tr[q][tx][4 * ty + 2] = t.z;
+      tr[q][tx][4 * ty + 3] = t.w;
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < GRED_G; ++q)
+    for (int q = 0; q < GRED_G; ++q) {
+      const float av[NK] = {a[q].x, a[q].y, a[q].z, a[q].w}, bv[NK] = {b[q].x, b[q].y, b[q].z, b[q].w},
+                  cv[NK] = {c1[q].x, c1[q].y, c1[q].z, c1[q].w};
 #pragma unroll
       for (int k = 0; k < NK; ++k) {
-        add2(rh[k], rl[k], a[q][k]);
-        add2(rh[k], rl[k], b[q][k]);
-        add2(ih[k], il[k], c1[q][k]);
-        add2(ih[k], il[k], -tr[q][tx][ty + 8 * k]);
+        add2(rh[k], rl[k], av[k]);
+        add2(rh[k], rl[k], bv[k]);
+        add2(ih[k], il[k], cv[k]);
+        add2(ih[k], il[k], -tr[q][4 * ty + k][tx]);
       }
+    }
     __syncthreads();
   }
   double2* Gl = G + (size_t)lf * C * C;
 #pragma unroll
   for (int k = 0; k < NK; ++k) {
-    const int c = c0 + ty + 8 * k;
+    const int cc = ccb + k;
     if (c < C && cc < C && c <= cc) {
       const double re = (double)rh[k] + (double)rl[k], im = (double)ih[k] + (double)il[k];
       if (c == cc) {

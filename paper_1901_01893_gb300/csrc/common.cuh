@@ -102,7 +102,7 @@ struct DevReport {
   int sweeps[SMSM_MAX_OUTER];
 };
 
-// The weights' quadrature (invsqrt.cu): W = wscale sum_j a_j ((G inv_c) + (shift + b_j) I)^(-1)
+// The weights' quadrature (invsqrt.cu): W = wscale sum_j a_j ((scale G inv_c) + (shift + b_j) I)^(-1)
 #define IS_MAXN 16  // terms at most
 #define IS_MAXQ 20  // largest condition number c/eps taken: 2^20
 struct IsRow {  // nodes for [2^-q, 1]
@@ -110,6 +110,7 @@ struct IsRow {  // nodes for [2^-q, 1]
   float a[IS_MAXN], b[IS_MAXN];
 };
 struct IsParam {  // one Hankel matrix's
+  float scale;  // power of two: the kernels hold scale G
   float inv_c, shift, wscale;
   int q, n;  // row of the table, terms (0: left to the eigensolver)
 };

@@ -45,16 +45,25 @@ __device__ __forceinline__ void ffma2(float2& acc, float2 a, float2 b) {
   acc = *reinterpret_cast<float2*>(&d);
 }
 
-// G in FP32, and each row's sum of |g| and of |g|^2: one warp per row
+// G in FP32, scaled by the power of two that brings its largest diagonal entry into [1, 2), and each row's
+// sum of |g| and of |g|^2: one warp per row.  (G has the square of the data's scale and is squared again from here
+// on: unscaled, data of 2^-45 or 2^30 times unit size left FP32's range.  A power of two changes no bits.)
 __global__ void __launch_bounds__(256) k_is_cvt(const double2* __restrict__ G, float2* __restrict__ G32,
-                                                float2* __restrict__ rows, int C) {
+                                                float2* __restrict__ rows, IsParam* __restrict__ prm, int C) {
   const int l = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= C) return;
   const size_t off = ((size_t)l * C + row) * C;
+  int e = -1023;  // largest exponent of the diagonal (-1023: all zero, 1024: not finite)
+  for (int j = lane; j < C; j += 32)
+    e = max(e, ((__double2hiint(G[((size_t)l * C + j) * C + j].x) >> 20) & 0x7ff) - 1023);
+  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  e = e == -1023 || e == 1024 ? 0 : min(max(e, -126), 126);
+  const float scale = __int_as_float((127 - e) << 23);
+  if (row == 0 && lane == 0) prm[l].scale = scale;
   float s1 = 0.f, s2 = 0.f;
   for (int j = lane; j < C; j += 32) {
     const double2 g = G[off + j];
-    const float2 v = cmk((float)g.x, (float)g.y);
+    const float2 v = cmk((float)g.x * scale, (float)g.y * scale);
     G32[off + j] = v;
     const float q = fmaf(v.x, v.x, v.y * v.y);
     s1 += sqrtf(q);
@@ -67,7 +76,7 @@ __global__ void __launch_bounds__(256) k_is_cvt(const double2* __restrict__ G, f
   if (lane == 0) rows[(size_t)l * C + row] = cmk(s1, s2);
 }
 
-// The squaring X X / tr(X)^2 of a Hermitian X, C x C, FP32.  A CTA computes a (16 R)^2 tile, a
+// The squaring X X / tr(X)^2 of a Hermitian X, C x C, FP32 (0 for X = 0: an empty slice).  A CTA computes a (16 R)^2 tile, a
 // thread R x R entries 16 apart, K in chunks fetched to registers one chunk ahead.  The left operand
 // is staged as (re, re, im, im), so that a complex multiply-add is two packed FMAs on loaded
 // registers: re x (b) and im x (b), summed apart and combined at the end.  R = 3 (48 x 48 tiles) when
@@ -121,7 +130,7 @@ __global__ void __launch_bounds__(256) k_is_square(const float2* __restrict__ X,
   t = 0.f;
 #pragma unroll
   for (int k = 0; k < 8; ++k) t += red[k];
-  const float sc = 1.f / t;
+  const float sc = t > 0.f ? 1.f / t : 0.f;  // (a NaN in X stays one)
   int s = 0;
   for (int k0 = 0; k0 < C; k0 += KT, s ^= 1) {
     const bool more = k0 + KT < C;
@@ -156,7 +165,7 @@ __global__ void __launch_bounds__(256) k_is_square(const float2* __restrict__ X,
     }
 }
 
-// largest eigenvalue of each G: tr(G S) / tr(S), S = the normalised 2^IS_SQ-th power
+// largest eigenvalue of each (scaled) G: tr(G S) / tr(S), S = the normalised 2^IS_SQ-th power; 0 for G = 0
 __global__ void __launch_bounds__(1024) k_is_lmax(const float2* __restrict__ G32, const float2* __restrict__ S,
                                                   float* __restrict__ lmax, int C) {
   __shared__ double num[32], den[32];
@@ -184,7 +193,7 @@ __global__ void __launch_bounds__(1024) k_is_lmax(const float2* __restrict__ G32
       dn += num[k];
       dd += den[k];
     }
-    lmax[l] = (float)(dn / dd);
+    lmax[l] = dd == 0.0 ? 0.f : (float)(dn / dd);
   }
 }
 
@@ -200,12 +209,12 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
   if (tid == 0) {
     SolverState* sd = st + d;
     if (outer == 0) {
-      float m = 0.f;
+      double m = 0.0;
       for (int l = 0; l < L; ++l) {
-        const float v = lmax[d * L + l];
+        const double v = (double)lmax[d * L + l] / prm[d * L + l].scale;
         m = v > m || v != v ? v : m;  // a NaN stays one
       }
-      sd->eps0 = eps0_rel * (double)m;
+      sd->eps0 = eps0_rel * m;
       sd->eps = sd->eps0;
       sd->eps_min = eps_min_rel * sd->eps0;
     } else {
@@ -237,20 +246,19 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
         m = fmaxf(m, mx[k]);
         q += sq[k];
       }
-      // c bounds the largest eigenvalue: row sums or the Frobenius norm (a little above, for rounding)
-      // (FP32: A = (G + eps I)/c whatever c is, as long as its parts use the same one)
-      const float eps = (float)eps_s;
-      const float c = 1.0001f * (fminf(m, sqrtf(q)) + eps);
-      IsParam p;
-      p.inv_c = 1.f / c;
-      p.shift = eps * p.inv_c;
-      p.wscale = sqrtf(p.inv_c);
+      // c bounds the largest eigenvalue of the scaled G: row sums or the Frobenius norm (a little above,
+      // for rounding); with eps > 0 an empty slice has c = eps and weight I/sqrt(eps)
+      IsParam p = prm[d * L + l];
+      const double eps = eps_s * p.scale, c = 1.0001 * ((double)fminf(m, sqrtf(q)) + eps);
+      p.inv_c = (float)(1.0 / c);
+      p.shift = (float)(eps * p.inv_c);
+      p.wscale = (float)sqrt((double)p.inv_c * p.scale);
       p.q = 0;
       p.n = 0;
-      const float cond = c / eps;
-      if (q > 0.f && eps > 0.f && cond <= (float)(1 << IS_MAXQ)) {  // false for NaN too
+      const double cond = c / eps;
+      if (q >= 0.f && c >= 1e-30 && cond <= (double)(1 << IS_MAXQ)) {  // false for NaN too
         int k = 0;
-        while ((float)(1 << k) < cond) ++k;
+        while ((double)(1 << k) < cond) ++k;
         p.q = k;
         p.n = tab[k].n;
       }
@@ -602,7 +610,7 @@ smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, co
   const int C = P->C, LD = P->LD, nb = rat_nb(C), nblk = nb * (nb + 1) / 2;
   if (T) T->begin(SMSM_STAGE_EIG);
   float2 *A = P->Gw, *Za = P->V, *Zb = P->Gw2;
-  k_is_cvt<<<dim3((C + 7) / 8, LD), 256, 0, s>>>(G, A, P->is_rows, C);
+  k_is_cvt<<<dim3((C + 7) / 8, LD), 256, 0, s>>>(G, A, P->is_rows, P->is_prm, C);
   SMSM_LAUNCH_CHECK("k_is_cvt");
   if (outer == 0) {
     const float2* X = A;

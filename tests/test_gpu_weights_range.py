@@ -1,0 +1,68 @@
+"""GPU: the IRLS weights (csrc/invsqrt.cu) over what a solve may meet: an empty slice, data of any scale.
+
+Tolerance: the FP32 whole-solve bar of test_gpu_parity.py, 2e-5 per slice, against the FP64 oracle.  The problem
+scales with its data when lambda does (W has the inverse scale), so one oracle solve serves every scale.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_1901_01893_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+SOLVE_TOL = 2e-5
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def smsm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1901_01893_gb300 import _build, smsm as mod
+
+    _build.build()
+    mod.lib()
+    return mod
+
+
+def c64(a):
+    return torch.from_numpy(np.ascontiguousarray(a).astype(np.complex64)).to(DEV)
+
+
+@pytest.mark.parametrize("Ns,r,N", [(4, 5, 64), (1, 4, 32), (8, 6, 48)])
+def test_an_empty_slice_leaves_the_others_alone(smsm, Ns, r, N):
+    # coil maps that are zero over a whole slice (all air): its Gram is exactly zero
+    g = synth.make_group(2, Ns, 6, N, 11)
+    S = g["sens"].copy()
+    S[1] = 0
+    _, y = O.make_data(dict(g, sens=S), 30.0)
+    y = y / np.sqrt(np.mean(np.abs(y) ** 2))
+    K, J, lam = 3, 3, 1e-2
+    rp = {}
+    ref = O.reconstruct(y, S, r, dict(K=K, J=J, lam=lam), report=rp)
+    p = smsm.Plan(2, Ns, 6, N, r)
+    p.set_sens(c64(S))
+    x, rep = p.reconstruct(c64(y), params=smsm.default_params(lam=lam, outer_iters=K, cg_iters=J))
+    x = x.cpu().numpy()
+    assert rep.status == 0
+    assert O.nrmse(x[0], ref[0]) < SOLVE_TOL
+    assert np.all(x[1] == 0)
+    assert rep.eps[0] == pytest.approx(rp["hist"][0]["eps"], rel=1e-5)
+
+
+@pytest.mark.parametrize("e", [-50, -45, -30, 0, 20, 30, 45, 55])
+def test_data_of_any_scale(smsm, e):
+    g = synth.make_group(2, 4, 6, 48, 12)
+    _, y = O.make_data(g, 30.0)
+    y = y / np.sqrt(np.mean(np.abs(y) ** 2))
+    K, J, lam, s = 3, 3, 1e-2, 2.0 ** e
+    rp = {}
+    ref = O.reconstruct(y, g["sens"], 5, dict(K=K, J=J, lam=lam), report=rp)
+    p = smsm.Plan(2, 4, 6, 48, 5)
+    p.set_sens(c64(g["sens"]))
+    x, rep = p.reconstruct(c64(y * s), params=smsm.default_params(lam=lam * s, outer_iters=K, cg_iters=J))
+    assert rep.status == 0 and list(rep.sweeps)[:K] == [0] * K
+    assert float(np.max(O.nrmse(x.cpu().numpy().astype(complex) / s, ref, axis=(1, 2, 3)))) < SOLVE_TOL
+    assert rep.eps[0] / s ** 2 == pytest.approx(rp["hist"][0]["eps"], rel=1e-5)

@@ -53,6 +53,11 @@ __global__ void __launch_bounds__(256) k_is_cvt(const double2* __restrict__ G, f
   const int l = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= C) return;
   const size_t off = ((size_t)l * C + row) * C;
+  constexpr int NV = (SMSM_MAX_C + 31) / 32;
+  double2 g[NV];  // the row's loads and the diagonal's in flight together
+#pragma unroll
+  for (int k = 0; k < NV; ++k)
+    if (lane + 32 * k < C) g[k] = G[off + lane + 32 * k];
   int e = -1023;  // largest exponent of the diagonal (-1023: all zero, 1024: not finite)
   for (int j = lane; j < C; j += 32)
     e = max(e, ((__double2hiint(G[((size_t)l * C + j) * C + j].x) >> 20) & 0x7ff) - 1023);
@@ -61,10 +66,11 @@ __global__ void __launch_bounds__(256) k_is_cvt(const double2* __restrict__ G, f
   const float scale = __int_as_float((127 - e) << 23);
   if (row == 0 && lane == 0) prm[l].scale = scale;
   float s1 = 0.f, s2 = 0.f;
-  for (int j = lane; j < C; j += 32) {
-    const double2 g = G[off + j];
-    const float2 v = cmk((float)g.x * scale, (float)g.y * scale);
-    G32[off + j] = v;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    if (lane + 32 * k >= C) break;
+    const float2 v = cmk((float)g[k].x * scale, (float)g[k].y * scale);
+    G32[off + lane + 32 * k] = v;
     const float q = fmaf(v.x, v.x, v.y * v.y);
     s1 += sqrtf(q);
     s2 += q;
@@ -82,7 +88,7 @@ __global__ void __launch_bounds__(256) k_is_cvt(const double2* __restrict__ G, f
 // registers: re x (b) and im x (b), summed apart and combined at the end.  R = 3 (48 x 48 tiles) when
 // the tiles fill the chip, R = 1 for a few matrices, where a CTA's serial K loop sets the time.
 template <int R>
-__global__ void __launch_bounds__(256) k_is_square(const float2* __restrict__ X, float2* __restrict__ out, int C) {
+__global__ void __launch_bounds__(256, R == 1 ? 5 : 1) k_is_square(const float2* __restrict__ X, float2* __restrict__ out, int C) {
   constexpr int T = 16 * R;
   constexpr int KT = R == 1 ? 48 : 16;
   constexpr int NE = (T * KT + 255) / 256;
@@ -203,15 +209,14 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
                                                   SolverState* st, DevReport* rep, IsParam* __restrict__ prm,
                                                   int* __restrict__ flag, const IsRow* __restrict__ tab, int L, int C,
                                                   int outer, double eps0_rel, double eta, double eps_min_rel) {
-  __shared__ float mx[8], sq[8];
   __shared__ double eps_s;
-  const int d = blockIdx.x, tid = threadIdx.x;
+  const int d = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     SolverState* sd = st + d;
     if (outer == 0) {
       double m = 0.0;
       for (int l = 0; l < L; ++l) {
-        const double v = (double)lmax[d * L + l] / prm[d * L + l].scale;
+        const double v = (double)lmax[d * L + l] * (double)__frcp_rn(prm[d * L + l].scale);  // (exact: a power of two)
         m = v > m || v != v ? v : m;  // a NaN stays one
       }
       sd->eps0 = eps0_rel * m;
@@ -222,10 +227,11 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
     }
     eps_s = sd->eps;
   }
-  for (int l = 0; l < L; ++l) {
+  __syncthreads();
+  for (int l = warp; l < L; l += 8) {  // a warp per slice
     const size_t off = (size_t)(d * L + l) * C;
     float m = 0.f, q = 0.f;
-    for (int j = tid; j < C; j += 256) {
+    for (int j = lane; j < C; j += 32) {
       const float2 v = rows[off + j];
       m = fmaxf(m, v.x);
       q += v.y;
@@ -234,31 +240,22 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
       m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
       q += __shfl_xor_sync(0xffffffffu, q, o);
     }
-    __syncthreads();
-    if ((tid & 31) == 0) {
-      mx[tid >> 5] = m;
-      sq[tid >> 5] = q;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      m = q = 0.f;
-      for (int k = 0; k < 8; ++k) {
-        m = fmaxf(m, mx[k]);
-        q += sq[k];
-      }
+    if (lane == 0) {
       // c bounds the largest eigenvalue of the scaled G: row sums or the Frobenius norm (a little above,
-      // for rounding); with eps > 0 an empty slice has c = eps and weight I/sqrt(eps)
+      // for rounding); with eps > 0 an empty slice has c = eps and weight I/sqrt(eps).  Whatever c
+      // rounds to, the shift and the final scale are of the same one.
       IsParam p = prm[d * L + l];
-      const double eps = eps_s * p.scale, c = 1.0001 * ((double)fminf(m, sqrtf(q)) + eps);
-      p.inv_c = (float)(1.0 / c);
+      const double eps = eps_s * p.scale;
+      const float c = (float)(1.0001 * ((double)fminf(m, sqrtf(q)) + eps));
+      p.inv_c = 1.f / c;
       p.shift = (float)(eps * p.inv_c);
-      p.wscale = (float)sqrt((double)p.inv_c * p.scale);
+      p.wscale = sqrtf(p.inv_c * p.scale);  // (the product is exact)
       p.q = 0;
       p.n = 0;
-      const double cond = c / eps;
-      if (q >= 0.f && c >= 1e-30 && cond <= (double)(1 << IS_MAXQ)) {  // false for NaN too
+      const float cond = c / (float)eps;
+      if (q >= 0.f && c >= 1e-30f && cond <= (float)(1 << IS_MAXQ)) {  // false for NaN too
         int k = 0;
-        while ((double)(1 << k) < cond) ++k;
+        while ((float)(1 << k) < cond) ++k;
         p.q = k;
         p.n = tab[k].n;
       }

@@ -26,7 +26,12 @@
 //
 // A matrix with c/eps above 2^IS_MAXQ (the start much smaller than the iterates, so that eps is
 // near G's FP32 rounding) is left to the eigensolver: is_flag is set and the Jacobi kernels, which
-// otherwise return at once, take it.
+// otherwise return at once, take it.  So is one whose elimination met a pivot below half its shift: every
+// pivot of a positive semidefinite G plus the shift is at least the shift, so the rounding of G or of the
+// elimination has then made it indefinite.  The eigensolver's weights clamp negative eigenvalues at 0; here they
+// stay what they are, which only the reduced-precision Gram makes matter: its three products leave out the
+// square of what a value loses to its first BF16 piece, up to 1.4e-5 of the largest eigenvalue.  There one more
+// elimination, of G + IS_PROBE eps I, says whether an eigenvalue lies below -IS_PROBE eps (it moves W by 3 %).
 #include <math.h>
 
 #include "common.cuh"
@@ -34,6 +39,7 @@
 
 #define IS_TOL 2e-7   // largest relative error of the quadrature
 #define IS_SQ 16      // squarings for the largest eigenvalue
+#define IS_PROBE 0.0625f
 #define RB 16         // block edge of the inverse
 
 // acc.x += a.x * b.x, acc.y += a.y * b.y in one instruction
@@ -88,7 +94,7 @@ __global__ void __launch_bounds__(256) k_is_cvt(const double2* __restrict__ G, f
 // registers: re x (b) and im x (b), summed apart and combined at the end.  R = 3 (48 x 48 tiles) when
 // the tiles fill the chip, R = 1 for a few matrices, where a CTA's serial K loop sets the time.
 template <int R>
-__global__ void __launch_bounds__(256, R == 1 ? 5 : 1) k_is_square(const float2* __restrict__ X, float2* __restrict__ out, int C) {
+__global__ void __launch_bounds__(256, R == 1 ? 5 : 3) k_is_square(const float2* __restrict__ X, float2* __restrict__ out, int C) {
   constexpr int T = 16 * R;
   constexpr int KT = R == 1 ? 48 : 16;
   constexpr int NE = (T * KT + 255) / 256;
@@ -298,11 +304,12 @@ __device__ __forceinline__ void rat_block(int b, int& i, int& j) {  // b = i (i 
 template <int SLOTS, int CL>
 __global__ void __launch_bounds__(32 * RAT_NW, 1)
     k_is_term(const float2* __restrict__ G32, const IsParam* __restrict__ prm, const IsRow* __restrict__ tab,
-              float2* __restrict__ part, int C, int nb, int l0) {
+              float2* __restrict__ part, int* __restrict__ flag, int C, int nb, int l0, int probes) {
   extern __shared__ __align__(16) float2 rsm[];
   const int task = blockIdx.x / CL, l = l0 + task / IS_MAXN, term = task % IS_MAXN;
   const IsParam pm = prm[l];
-  if (term >= pm.n) return;  // every CTA of a cluster alike
+  const bool probe = probes && pm.n > 0 && term == pm.n;
+  if (term >= pm.n && !probe) return;  // every CTA of a cluster alike
   const int ld = RB * nb + 2;
   float2* Bf = rsm;                                   // [1 or 2][RB][ld]
   float2* Q = rsm + (CL > 1 ? 2 : 1) * RB * ld;       // [RB][ld]
@@ -311,7 +318,8 @@ __global__ void __launch_bounds__(32 * RAT_NW, 1)
   const int rank = CL > 1 ? (int)cl_rank() : 0;
   const int r0 = (lane >> 3) * 4, c0 = (lane & 7) * 2;
   const int nblk = nb * (nb + 1) / 2;
-  const float shift = pm.shift + tab[pm.q].b[term];
+  const float shift = probe ? IS_PROBE * pm.shift : pm.shift + tab[pm.q].b[term];
+  const float most = probe ? 3e38f : rsqrtf(0.5f * shift);  // of 1/sqrt(pivot)
   const float2* Gl = G32 + (size_t)l * C * C;
   float2 R[SLOTS][4][2];
   int bi[SLOTS], bj[SLOTS];
@@ -338,6 +346,7 @@ __global__ void __launch_bounds__(32 * RAT_NW, 1)
         R[s][u][v] = g;
       }
   }
+  bool bad = false;  // (warp 1) a pivot was not what a positive definite matrix has
   if (CL > 1) cl_sync();  // every CTA runs before any writes into another's shared memory
   for (int k = 0; k < nb; ++k) {
     float2* Bk = Bf + (CL > 1 ? (k & 1) * RB * ld : 0);
@@ -392,6 +401,8 @@ __global__ void __launch_bounds__(32 * RAT_NW, 1)
       }
     }
     __syncthreads();
+    // D's diagonal: 1/sqrt(pivot), a NaN where it is negative (looked at here, off the pivot block's chain)
+    if (warp == 1 && lane < RB && k * RB + lane < C) bad |= !(D[lane * (RB + 2)].x <= most);
     for (int e = tid; e < RB * nb * 4; e += 32 * RAT_NW) {
       const int rg = e / (RB * nb), col = e - rg * RB * nb;  // four rows of one column
       float2 q[4];
@@ -413,7 +424,7 @@ __global__ void __launch_bounds__(32 * RAT_NW, 1)
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < SLOTS; ++s) {
-      if (bi[s] < 0) continue;
+      if (bi[s] < 0 || (probe && bj[s] <= k)) continue;  // (the probe needs the trailing matrix only)
       const float2* qi = Q + bi[s] * RB + r0;
       const float2* qj = Q + bj[s] * RB + c0;
       float2 t[4][2];
@@ -439,6 +450,8 @@ __global__ void __launch_bounds__(32 * RAT_NW, 1)
           R[s][u][v] = cmk(fmaf(sg, t[u][v].x, R[s][u][v].x), fmaf(sg, t[u][v].y, R[s][u][v].y));
     }
   }
+  if (bad) atomicOr(flag + l, 1);
+  if (probe) return;
   const float w = tab[pm.q].a[term];
   float2* out = part + ((size_t)(l - l0) * IS_MAXN + term) * nblk * (RB * RB);
 #pragma unroll
@@ -510,7 +523,7 @@ static std::vector<IsRow> make_table() {
       x = t;
     }
     const double K = M_PI / (2.0 * x);
-    for (int n = 2; n <= IS_MAXN; ++n) {
+    for (int n = 2; n < IS_MAXN; ++n) {  // (one slot is the probe's)
       double a[IS_MAXN], b[IS_MAXN], worst = 0.0;
       for (int j = 0; j < n; ++j) {
         double sn, cn, dn;
@@ -559,7 +572,7 @@ size_t invsqrt_per(const smsm_plan_s* P) {  // complex values of one matrix's te
   return (size_t)IS_MAXN * (nb * (nb + 1) / 2) * RB * RB;
 }
 
-typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int, int, int);
+typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int*, int, int, int, int);
 
 // Slots = blocks per warp.  One CTA's 16 warps hold up to 5 blocks each (C <= 192: 80 of 128 registers);
 // above, four CTAs hold the 105 (C = 208+) to 210 (C = 320) blocks with 2 to 4 each.
@@ -644,7 +657,8 @@ smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, co
     cfg.attrs = at;
     cfg.numAttrs = 1;
     SMSM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, (const float2*)A, (const IsParam*)P->is_prm, (const IsRow*)P->is_tab,
-                                     P->scratch, C, nb, l0));
+                                     P->scratch, P->is_flag, C, nb, l0,
+                                     (int)(P->precision == SMSM_PRECISION_BF16_SPLIT)));
     k_is_sum<<<dim3(nblk, n), RB * RB, 0, s>>>(P->scratch, P->Wf, P->is_prm, C, nblk, l0);
     SMSM_LAUNCH_CHECK("k_is_sum");
   }

@@ -66,3 +66,29 @@ def test_data_of_any_scale(smsm, e):
     assert rep.status == 0 and list(rep.sweeps)[:K] == [0] * K
     assert float(np.max(O.nrmse(x.cpu().numpy().astype(complex) / s, ref, axis=(1, 2, 3)))) < SOLVE_TOL
     assert rep.eps[0] / s ** 2 == pytest.approx(rp["hist"][0]["eps"], rel=1e-5)
+
+
+@pytest.mark.parametrize("eps0", [1e-5, 1.2e-5, 2e-5, 1e-4])
+def test_an_indefinite_gram_takes_the_eigensolver(smsm, eps0):
+    # BF16 split Gram of shots that are constants 1.0078125 +- 0.0038 over k-space: the part each value loses to the
+    # first BF16 piece alternates in sign over the shots, so it is coherent and orthogonal to the data; three products
+    # leave out its square, -1.4e-5 of the largest eigenvalue: more than eps, or a part of it.  The eigensolver clamps it.
+    # The bar: no further from the oracle than the solve that uses the eigensolver throughout (its own error there is
+    # rounding next to eps), with the short solve's bar on top.
+    v = 1.0078125 + 0.0038 * np.array([1, -1] * 4)
+    x0 = np.ones((1, 8, 64, 64)) * v[None, :, None, None] * (1 + 0j)
+    g = synth.make_group(1, 8, 4, 64, 3)
+    _, y = O.make_data(g, 30.0)
+    y = y / np.sqrt(np.mean(np.abs(y) ** 2))
+    par = dict(eps0_rel=eps0, eps_min_rel=1.0)
+    ref = O.reconstruct(y, g["sens"], 2, dict(K=1, J=2, lam=1e-1, **par), x0=x0)
+    p = smsm.Plan(1, 8, 4, 64, 2, precision=smsm.SMSM_PRECISION_BF16_SPLIT)
+    p.set_sens(c64(g["sens"]))
+    err = {}
+    for cold in (0, 1):
+        prm = smsm.default_params(lam=1e-1, outer_iters=1, cg_iters=2, warm=1, eig_cold=cold, **par)
+        x, rep = p.reconstruct(c64(y), x=c64(x0), params=prm)
+        assert rep.status == 0
+        err[cold] = float(np.max(O.nrmse(x.cpu().numpy(), ref, axis=(1, 2, 3))))
+    print("errors", err)
+    assert err[0] < 2 * err[1] + SOLVE_TOL

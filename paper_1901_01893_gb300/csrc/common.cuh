@@ -109,6 +109,8 @@ struct IsRow {  // nodes for [2^-q, 1]
   int n;
   float a[IS_MAXN], b[IS_MAXN];
 };
+#define IS_EIG 1   // this matrix's weight comes from the eigensolver
+#define IS_WARM 2  // which starts from the eigenvectors of the outer iteration before
 struct IsParam {  // one Hankel matrix's
   float scale;  // power of two: the kernels hold scale G
   float inv_c, shift, wscale;
@@ -168,7 +170,7 @@ struct smsm_plan_s {
   IsParam* is_prm;   // [LD]
   IsRow* is_tab;     // [IS_MAXQ + 1]
   float2* scratch;   // per matrix: the Gram's lagged sums, then the weights' terms (scratch_count)
-  int* is_flag;      // [LD] 1: this matrix's weight comes from the eigensolver
+  int* is_flag;      // [LD] IS_EIG | IS_WARM
   float2* wper;      // [L][Ns][Ns][R2*R2]
   float2* wcls;      // [LD][R2*R2 classes][Ns (i')][R2*R2 taps][Ns (i)] border correction taps
   float2* multT;     // [L][Ns(Ns+1)/2][N(x)][N(y)]: upper triangle of the Hermitian shot coupling
@@ -341,15 +343,15 @@ size_t eig_jacobi_smem(int Cp);
 bool eig_pair_supported(int Cp);
 bool eig_cluster_supported(int C);
 smsm_status eig_cluster_init_attrs(int C);
-smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const float2* T, int max_sweeps, float tol,
-                               float floor_rel, const int* only, cudaStream_t s);
+smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const float2* T, float2* V, int max_sweeps,
+                               float tol, float floor_rel, const int* only, cudaStream_t s);
 // invsqrt.cu
 const std::vector<IsRow>& invsqrt_table();
 size_t invsqrt_per(const smsm_plan_s* P);
 smsm_status invsqrt_init_attrs(const smsm_plan_s* P);
 bool invsqrt_applies(const smsm_plan_s* P, const smsm_params* prm);
-smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, const smsm_params* prm, cudaStream_t s,
-                           Timer* T);
+smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, const float2* V, int outer, const smsm_params* prm,
+                           cudaStream_t s, Timer* T);
 smsm_status operators_init_attrs();
 size_t smsm_col_smem_bytes(const smsm_plan_s* P);
 int band_blocks(const smsm_plan_s* P);

@@ -92,10 +92,14 @@ __host__ __device__ inline size_t jac_region_a(int Cp) { return (((size_t)Cp * (
 __host__ __device__ inline size_t jac_smem_bytes(int Cp) { return jac_region_a(Cp) + (size_t)(Cp / 2) * 32; }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(1024)
-    k_jacobi(const double2* __restrict__ G, const float2* __restrict__ Gw, float* __restrict__ eig,
+    k_jacobi(const double2* __restrict__ G, const float2* Gw, float* __restrict__ eig,
              float2* __restrict__ V, int warmv, int* __restrict__ sweeps_out, int C, int Cp, int max_sweeps, float tol,
              float floor_rel, SolverState* st, int L, int* __restrict__ errflag, const int* __restrict__ only) {
-  if (only && !only[blockIdx.x >> 1]) return;  // both CTAs of the cluster alike
+  if (only) {  // IS_EIG, IS_WARM; both CTAs of the cluster alike
+    const int take = only[blockIdx.x >> 1];
+    if (!(take & IS_EIG)) return;
+    if (!(take & IS_WARM)) Gw = nullptr, warmv = 0;
+  }
   extern __shared__ __align__(16) unsigned char jsm[];
   __shared__ __align__(8) uint64_t full_b[2], empty_b[2];
   __shared__ int hdr[2];
@@ -392,7 +396,7 @@ __global__ void __launch_bounds__(256) k_cgemm(const double2* __restrict__ G, co
                                                const float* __restrict__ eig, const SolverState* __restrict__ st,
                                                int Cp, int mode, int rank, int L, const int* __restrict__ only, int* rep_sweeps,
                                                const int* __restrict__ sweeps) {
-  if (only && !only[blockIdx.z]) return;
+  if (only && !(only[blockIdx.z] & IS_EIG)) return;
   // the report follows direction 0: its slices are matrices 0 .. L - 1
   if (OP == SG_W && rep_sweeps && blockIdx.z < L && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
     atomicMax(rep_sweeps, sweeps[blockIdx.z]);
@@ -572,21 +576,24 @@ smsm_status launch_eig_weights(const smsm_plan_s* P, const double2* G, int outer
   const int warm = (outer > 0 && !prm->eig_cold) ? 1 : 0;
   smsm_status sg;
   if (invsqrt_applies(P, prm)) {
-    if ((sg = launch_invsqrt(P, G, outer, prm, s, T))) return sg;
-    // the matrices it left: eigenvectors from scratch, V re-orthonormalised, W (the launches
-    // return at once for every other matrix)
+    // V, where the eigenvectors are, and V2, where the re-orthonormalised ones go, change places from one
+    // outer iteration to the next
+    float2 *V = outer & 1 ? P->Gw2 : P->V, *V2 = outer & 1 ? P->V : P->Gw2;
+    if ((sg = launch_invsqrt(P, G, V, outer, prm, s, T))) return sg;
+    // the matrices it left: eigenvectors (the weights' kernels left the warm start's product in Gw), V
+    // re-orthonormalised, W (the launches return at once for every other matrix)
     const int* only = P->is_flag;
     if (T) T->begin(SMSM_STAGE_VAPPLY);
     if (P->eig_cluster) {
-      if ((sg = launch_eig_cluster(P, G, nullptr, msw, 2e-6f, 1e-12f, only, s))) return sg;
+      if ((sg = launch_eig_cluster(P, G, P->Gw, V, msw, 2e-6f, 1e-12f, only, s))) return sg;
     } else {
-      k_jacobi<<<2 * P->LD, 1024, jac_smem_bytes(Cp), s>>>(G, nullptr, P->eig, P->V, 0, P->sweeps, C, Cp, msw, 1e-6f,
+      k_jacobi<<<2 * P->LD, 1024, jac_smem_bytes(Cp), s>>>(G, P->Gw, P->eig, V, 1, P->sweeps, C, Cp, msw, 1e-6f,
                                                             1e-12f, P->st, P->L, P->devflag, only);
       SMSM_LAUNCH_CHECK("k_jacobi");
     }
-    if ((sg = launch_cgemm<SG_VHV>(P, nullptr, P->V, nullptr, P->Gw, prm, s, only))) return sg;
-    if ((sg = launch_cgemm<SG_NS>(P, nullptr, P->V, P->Gw, P->Gw2, prm, s, only))) return sg;
-    if ((sg = launch_cgemm<SG_W>(P, nullptr, P->Gw2, nullptr, P->Wf, prm, s, only,
+    if ((sg = launch_cgemm<SG_VHV>(P, nullptr, V, nullptr, P->Gw, prm, s, only))) return sg;
+    if ((sg = launch_cgemm<SG_NS>(P, nullptr, V, P->Gw, V2, prm, s, only))) return sg;
+    if ((sg = launch_cgemm<SG_W>(P, nullptr, V2, nullptr, P->Wf, prm, s, only,
                                   outer < SMSM_MAX_OUTER ? P->rep->sweeps + outer : nullptr)))
       return sg;
     if (T) T->end(SMSM_STAGE_VAPPLY);
@@ -597,7 +604,7 @@ smsm_status launch_eig_weights(const smsm_plan_s* P, const double2* G, int outer
     // one-sided Jacobi on A = G V_prev (the congruence's first product) or on G itself
     if (warm && (sg = launch_cgemm<SG_GV>(P, G, P->V, nullptr, P->Gw, prm, s))) return sg;
     const float tol = prm->eig_tol > 0.f ? prm->eig_tol : 2e-6f;
-    smsm_status st = launch_eig_cluster(P, G, warm ? P->Gw : nullptr, msw, tol, 1e-12f, nullptr, s);
+    smsm_status st = launch_eig_cluster(P, G, warm ? P->Gw : nullptr, P->V, msw, tol, 1e-12f, nullptr, s);
     if (st) return st;
   } else {
   if (warm) {

@@ -140,10 +140,14 @@ __device__ __forceinline__ void osj_move(float2* sm, int F4, uint32_t rank, int 
 
 template <int KR>
 __global__ void __cluster_dims__(OSJ_R, 1, 1) __launch_bounds__(640, 1)
-    k_jacobi_os(const double2* __restrict__ G, const float2* __restrict__ T, float* __restrict__ eig,
+    k_jacobi_os(const double2* __restrict__ G, const float2* T, float* __restrict__ eig,
                 float2* __restrict__ V, int* __restrict__ sweeps_out, int C, int Cp, int max_sweeps, float tol,
                 float floor_rel, SolverState* st, int L, const int* __restrict__ only) {
-  if (only && !only[blockIdx.x / OSJ_R]) return;  // every CTA of the cluster alike
+  if (only) {  // IS_EIG, IS_WARM; every CTA of the cluster alike
+    const int take = only[blockIdx.x / OSJ_R];
+    if (!(take & IS_EIG)) return;
+    if (!(take & IS_WARM)) T = nullptr;
+  }
   extern __shared__ __align__(16) float2 osm[];
   __shared__ int vote[OSJ_R];
   __shared__ float dmax_s;
@@ -302,12 +306,12 @@ smsm_status eig_cluster_init_attrs(int C) {
   return SMSM_OK;
 }
 
-smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const float2* T, int max_sweeps, float tol,
-                               float floor_rel, const int* only, cudaStream_t s) {
+smsm_status launch_eig_cluster(const smsm_plan_s* P, const double2* G, const float2* T, float2* V, int max_sweeps,
+                               float tol, float floor_rel, const int* only, cudaStream_t s) {
   OsjFn fn = osj_fn(P->C);
   if (!fn) return SMSM_ERR_ARG;
-  fn<<<OSJ_R * P->LD, 32 * osj_w(P->C), osj_smem(P->C), s>>>(G, T, P->eig, P->V, P->sweeps, P->C, P->Cp, max_sweeps,
-                                                             tol, floor_rel, P->st, P->L, only);
+  fn<<<OSJ_R * P->LD, 32 * osj_w(P->C), osj_smem(P->C), s>>>(G, T, P->eig, V, P->sweeps, P->C, P->Cp, max_sweeps, tol,
+                                                             floor_rel, P->st, P->L, only);
   SMSM_LAUNCH_CHECK("k_jacobi_os");
   return SMSM_OK;
 }

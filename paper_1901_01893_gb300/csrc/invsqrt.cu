@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(256) k_is_sched(const float2* __restrict__ row
         p.q = k;
         p.n = tab[k].n;
       }
-      flag[d * L + l] = p.n == 0;
+      const int had = outer > 0 ? flag[d * L + l] & IS_EIG : 0;  // the eigenvectors before this are there
+      flag[d * L + l] = p.n > 0 ? 0 : (had ? IS_EIG | IS_WARM : IS_EIG);
       prm[d * L + l] = p;
     }
   }
@@ -301,15 +302,35 @@ __device__ __forceinline__ void rat_block(int b, int& i, int& j) {  // b = i (i 
   j = b - i * (i + 1) / 2;
 }
 
+// The warm start of a matrix left to the eigensolver, by the CTAs its terms and their sum would have had (own
+// launches would cost every solve their latency): T = G V here, from the eigenvectors of the outer
+// iteration before, V^H T (two-CTA solver) or T itself (cluster solver) in k_is_sum.
+__device__ __noinline__ void is_gv(const float2* __restrict__ G32, const float2* __restrict__ V, float2* __restrict__ T,
+                                   float inv_scale, int C, int share, int shares) {
+  for (int e = share * blockDim.x + threadIdx.x; e < C * C; e += shares * blockDim.x) {
+    const int a = e / C, b = e - a * C;
+    float2 t = cmk(0.f, 0.f);
+    for (int k = 0; k < C; ++k) cfma(t, G32[(size_t)a * C + k], V[(size_t)k * C + b]);
+    T[e] = cscale(t, inv_scale);
+  }
+}
+
 template <int SLOTS, int CL>
 __global__ void __launch_bounds__(32 * RAT_NW, 1)
     k_is_term(const float2* __restrict__ G32, const IsParam* __restrict__ prm, const IsRow* __restrict__ tab,
-              float2* __restrict__ part, int* __restrict__ flag, int C, int nb, int l0, int probes) {
+              float2* __restrict__ part, int* __restrict__ flag, const float2* __restrict__ V, int C, int nb, int l0,
+              int probes) {
   extern __shared__ __align__(16) float2 rsm[];
   const int task = blockIdx.x / CL, l = l0 + task / IS_MAXN, term = task % IS_MAXN;
   const IsParam pm = prm[l];
   const bool probe = probes && pm.n > 0 && term == pm.n;
-  if (term >= pm.n && !probe) return;  // every CTA of a cluster alike
+  if (term >= pm.n && !probe) {  // every CTA of a cluster alike
+    if (pm.n == 0 && (flag[l] & IS_WARM))
+      is_gv(G32 + (size_t)l * C * C, V + (size_t)l * C * C,
+            part + (size_t)(l - l0) * IS_MAXN * (nb * (nb + 1) / 2) * (RB * RB), __frcp_rn(pm.scale), C,
+            blockIdx.x % (IS_MAXN * CL), IS_MAXN * CL);
+    return;
+  }
   const int ld = RB * nb + 2;
   float2* Bf = rsm;                                   // [1 or 2][RB][ld]
   float2* Q = rsm + (CL > 1 ? 2 : 1) * RB * ld;       // [RB][ld]
@@ -466,14 +487,34 @@ __global__ void __launch_bounds__(32 * RAT_NW, 1)
 }
 
 // W = c^(-1/2) times the sum of the terms (fixed order); the upper triangle mirrors the lower
+// (for a matrix left to the eigensolver: its warm start's matrix into Gw, see is_gv)
 __global__ void __launch_bounds__(RB* RB) k_is_sum(const float2* __restrict__ part, float2* __restrict__ W,
-                                                   const IsParam* __restrict__ prm, int C, int nblk, int l0) {
+                                                   const IsParam* __restrict__ prm, const int* __restrict__ flag,
+                                                   const float2* __restrict__ V, float2* __restrict__ Gw, int one_sided,
+                                                   int C, int nblk, int l0) {
   __shared__ float2 t[RB][RB + 1];
   const int l = l0 + blockIdx.y, b = blockIdx.x, tid = threadIdx.x, r = tid / RB, c = tid % RB;
   const int n = prm[l].n;
-  if (n == 0) return;
   int i, j;
   rat_block(b, i, j);
+  if (n == 0) {
+    if (!(flag[l] & IS_WARM)) return;
+    const float2* T = part + (size_t)blockIdx.y * IS_MAXN * nblk * (RB * RB);
+    const float2* Vl = V + (size_t)l * C * C;
+    float2* out = Gw + (size_t)l * C * C;
+    const int a = i * RB + r, bb = j * RB + c;  // of the lower triangle's blocks
+    if (a >= C || bb >= C) return;
+    if (one_sided) {
+      out[(size_t)a * C + bb] = T[(size_t)a * C + bb];
+      out[(size_t)bb * C + a] = T[(size_t)bb * C + a];
+    } else if (bb <= a) {  // the eigensolver takes the mean of an entry and its mirror's conjugate
+      float2 s = cmk(0.f, 0.f);
+      for (int k = 0; k < C; ++k) cfmacj(s, Vl[(size_t)k * C + a], T[(size_t)k * C + bb]);
+      out[(size_t)a * C + bb] = s;
+      out[(size_t)bb * C + a] = conjf2(s);
+    }
+    return;
+  }
   float2 s = cmk(0.f, 0.f);
   const float2* p = part + ((size_t)blockIdx.y * IS_MAXN * nblk + b) * (RB * RB) + tid;
   for (int k = 0; k < n; ++k) s = cadd(s, p[(size_t)k * nblk * (RB * RB)]);
@@ -572,7 +613,7 @@ size_t invsqrt_per(const smsm_plan_s* P) {  // complex values of one matrix's te
   return (size_t)IS_MAXN * (nb * (nb + 1) / 2) * RB * RB;
 }
 
-typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int*, int, int, int, int);
+typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int*, const float2*, int, int, int, int);
 
 // Slots = blocks per warp.  One CTA's 16 warps hold up to 5 blocks each (C <= 192: 80 of 128 registers);
 // above, four CTAs hold the 105 (C = 208+) to 210 (C = 320) blocks with 2 to 4 each.
@@ -615,8 +656,9 @@ smsm_status invsqrt_init_attrs(const smsm_plan_s* P) {
   return SMSM_OK;
 }
 
-smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, const smsm_params* prm, cudaStream_t s,
-                           Timer* T) {
+// V: where the eigenvectors of matrices left to the eigensolver in the outer iteration before are
+smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, const float2* V, int outer, const smsm_params* prm,
+                           cudaStream_t s, Timer* T) {
   const int C = P->C, LD = P->LD, nb = rat_nb(C), nblk = nb * (nb + 1) / 2;
   if (T) T->begin(SMSM_STAGE_EIG);
   float2 *A = P->Gw, *Za = P->V, *Zb = P->Gw2;
@@ -657,9 +699,10 @@ smsm_status launch_invsqrt(const smsm_plan_s* P, const double2* G, int outer, co
     cfg.attrs = at;
     cfg.numAttrs = 1;
     SMSM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, (const float2*)A, (const IsParam*)P->is_prm, (const IsRow*)P->is_tab,
-                                     P->scratch, P->is_flag, C, nb, l0,
+                                     P->scratch, P->is_flag, V, C, nb, l0,
                                      (int)(P->precision == SMSM_PRECISION_BF16_SPLIT)));
-    k_is_sum<<<dim3(nblk, n), RB * RB, 0, s>>>(P->scratch, P->Wf, P->is_prm, C, nblk, l0);
+    k_is_sum<<<dim3(nblk, n), RB * RB, 0, s>>>(P->scratch, P->Wf, P->is_prm, P->is_flag, V, P->Gw, P->eig_cluster, C,
+                                                nblk, l0);
     SMSM_LAUNCH_CHECK("k_is_sum");
   }
   if (T) T->end(SMSM_STAGE_EIG);

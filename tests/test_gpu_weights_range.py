@@ -92,3 +92,28 @@ def test_an_indefinite_gram_takes_the_eigensolver(smsm, eps0):
         err[cold] = float(np.max(O.nrmse(x.cpu().numpy(), ref, axis=(1, 2, 3))))
     print("errors", err)
     assert err[0] < 2 * err[1] + SOLVE_TOL
+
+
+@pytest.mark.parametrize("Ns,r,N", [(4, 4, 32), (4, 6, 48), (8, 6, 48)])
+def test_matrices_left_to_the_eigensolver_start_warm(smsm, Ns, r, N):
+    # a start 1e-3 of the data's size: from the second outer iteration on c/eps is beyond the quadrature's range, and
+    # from the third on the eigensolver has the eigenvectors of the iteration before.  Fewer sweeps than from scratch
+    # in every one of them, and no further from the oracle (the bar of the test next to this in test_gpu_weights.py).
+    g = synth.make_group(2, Ns, 6, N, 4)
+    _, y = O.make_data(g, 30.0)
+    y = y / np.sqrt(np.mean(np.abs(y) ** 2))
+    x0 = O.adjoint(y, g["sens"], 2) * 1e-3
+    K, J, lam = 6, 3, 1e-3
+    ref = O.reconstruct(y, g["sens"], r, dict(K=K, J=J, lam=lam), x0=x0)
+    p = smsm.Plan(2, Ns, 6, N, r)
+    p.set_sens(c64(g["sens"]))
+    err, sweeps = {}, {}
+    for cold in (0, 1):
+        prm = smsm.default_params(lam=lam, outer_iters=K, cg_iters=J, warm=1, eig_cold=cold)
+        x, rep = p.reconstruct(c64(y), x=c64(x0), params=prm)
+        assert rep.status == 0
+        err[cold], sweeps[cold] = float(np.max(O.nrmse(x.cpu().numpy(), ref, axis=(1, 2, 3)))), list(rep.sweeps)[:K]
+    print("errors", err, "sweeps", sweeps)
+    assert sweeps[0][0] == 0 and sweeps[0][1] > 0
+    assert all(a < b for a, b in zip(sweeps[0][2:], sweeps[1][2:]))
+    assert err[0] < 2 * err[1] + SOLVE_TOL

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
   }
 
   // partial of Re<img, acc> (Parseval: equals Re<p, q> in k-space)
-  float ds = 0.f;  // FP32 over this lane's few pixels, FP64 from there on
+  float dh = 0.f, dl = 0.f;  // high and low parts
 #pragma unroll
   for (int l = 0; l < L; ++l)
 #pragma unroll
@@ -211,10 +211,11 @@ __global__ void __launch_bounds__(256) k_col_fast(ColArgs a) {
         for (int j = 0; j < Ns; ++j) cfma(q, mult_at(ml, i, j, Ns, NN, (size_t)x * N + y), img[(l * Ns + j) * N + y]);
         acc[l][k] = cmk(fmaf(a.lambda, q.x, acc[l][k].x), fmaf(a.lambda, q.y, acc[l][k].y));
       }
-      ds = fmaf(u.x, acc[l][k].x, fmaf(u.y, acc[l][k].y, ds));
+      add2_prod(dh, dl, u.x, acc[l][k].x);
+      add2_prod(dh, dl, u.y, acc[l][k].y);
       tmp[(l * Ns + i) * N + y] = cscale(acc[l][k], sgn_par(y));
     }
-  double dsum = ds;
+  double dsum = (double)dh + (double)dl;
   for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
   if (lane == 0) red[warp] = dsum;
   __syncthreads();

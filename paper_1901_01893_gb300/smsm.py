@@ -115,6 +115,8 @@ def lib() -> ctypes.CDLL:
     L.smsm_cnn_create.restype = st
     L.smsm_cnn_destroy.argtypes = [vp]
     L.smsm_cnn_destroy.restype = st
+    L.smsm_cnn_device_status.argtypes = [vp, vp]
+    L.smsm_cnn_device_status.restype = st
     L.smsm_cnn_param_count.argtypes = [vp]
     L.smsm_cnn_param_count.restype = ctypes.c_size_t
     for fn in ("smsm_cnn_set_params", "smsm_cnn_get_params"):
@@ -358,6 +360,10 @@ class CNN:
             self.close()
         except Exception:
             pass
+
+    def device_status(self) -> int:
+        """Synchronise, return the network's device error flag (0 = fine) and clear it."""
+        return lib().smsm_cnn_device_status(self._h, _stream())
 
     def _io(self, t: torch.Tensor, n: int, name: str) -> int:
         return _dev(t, (n, self.B, self.H, self.W), name)

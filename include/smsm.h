@@ -292,7 +292,8 @@ smsm_status smsm_reconstruct_groups(int n, smsm_plan_t const* plans, const void*
  * image domain, or phase == NULL for no phase correction) and the slices are unfolded
  * by least squares: cg_iters steps of CG on A^H A x = A^H y from x = 0.
  *   y: [D][Ns][Nc][N/Ns][N] complex64; x: [D][L][1][N][N] complex64 (overwritten).
- * Runs on the stream without a graph; `report` (nullable) gets the status after a sync.
+ * Runs on the stream without a graph; `report` (nullable) gets the status after a sync,
+ * the plan's device error flag included.
  */
 smsm_status smsm_sense(smsm_plan_t plan, const void* y, const void* phase, void* x, int cg_iters,
                        smsm_report* report, void* stream);
@@ -407,7 +408,7 @@ smsm_status smsm_learned_start(smsm_plan_t plan, smsm_cnn_t cnn, const void* x_i
 /*
  * Synchronise `stream` and report the plan's device error flag: SMSM_OK, or
  * SMSM_ERR_TIMEOUT when a kernel gave up a bounded wait (its outputs are then
- * unspecified).  smsm_reconstruct's report carries the same flag.
+ * unspecified).  The reports of smsm_reconstruct and smsm_sense carry the same flag.
  */
 smsm_status smsm_plan_device_status(smsm_plan_t plan, void* stream);
 

@@ -828,10 +828,13 @@ smsm_status solver_sense(smsm_plan_s* P, const void* y, const void* phase, void*
   SMSM_CUDA_TRY(cudaMemcpyAsync(x, P->xs, sizeof(float2) * nx, cudaMemcpyDeviceToDevice, s));
   if (report) {
     std::vector<SolverState> hs(P->D);
+    int flag = 0;  // raised by the column stage where a wait for its copies ran out
     SMSM_CUDA_TRY(cudaMemcpyAsync(hs.data(), P->st, sizeof(SolverState) * P->D, cudaMemcpyDeviceToHost, s));
+    SMSM_CUDA_TRY(cudaMemcpyAsync(&flag, P->devflag, sizeof(int), cudaMemcpyDeviceToHost, s));
     SMSM_CUDA_TRY(cudaStreamSynchronize(s));
     memset(report, 0, sizeof(*report));
     for (int d = 0; d < P->D && !report->status; ++d) report->status = hs[d].status;
+    if (!report->status && flag) report->status = flag;
     report->lanes = 1;
     report->lane0_batch = P->D;
   }

@@ -41,3 +41,14 @@ def test_network_reports_and_clears_its_flag(smsm):
     assert e.value.status == smsm.SMSM_ERR_TIMEOUT
     loss, _ = net.gradients(a, a)
     assert loss > 0
+
+
+def test_reports_carry_the_plans_flag(smsm):
+    p = smsm.Plan(1, 2, 2, 32, 2)
+    p.set_sens(torch.randn(1, 2, 32, 32, dtype=torch.complex64, device=DEV))
+    y = torch.randn(p.y_shape, dtype=torch.complex64, device=DEV)
+    assert p.sense(y, cg_iters=2)[1].status == 0
+    smsm.lib().smsm_plan_raise_for_test(p._h, smsm.SMSM_ERR_TIMEOUT)
+    assert p.sense(y, cg_iters=2)[1].status == smsm.SMSM_ERR_TIMEOUT
+    assert p.reconstruct(y)[1].status == smsm.SMSM_ERR_TIMEOUT
+    assert p.device_status() == smsm.SMSM_ERR_TIMEOUT

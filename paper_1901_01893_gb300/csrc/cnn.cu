@@ -135,6 +135,20 @@ __device__ __forceinline__ bool cv_wait(uint64_t* mbar, uint32_t parity, volatil
   return false;
 }
 
+// Two floats in BF16 (lo in the low half).  The first two pieces saturate: a finite value above the largest BF16 one
+// leaves a remainder that the other pieces hold, and an infinite one goes to the third piece, where inf - inf would
+// make a remainder a NaN.
+__device__ __forceinline__ uint32_t cv_pack_sat(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
+}
+__device__ __forceinline__ uint32_t cv_pack(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
+}
+
 __host__ __device__ inline uint32_t cv_a_bytes(const ConvShape& g) {  // one piece of one stage
   return 2u * (uint32_t)(CV_TL + 2 * g.P + 2) * 16u;
 }
@@ -218,13 +232,14 @@ __global__ void __launch_bounds__(CV_THREADS, 1)
         }
 #pragma unroll
         for (int piece = 0; piece < 3; ++piece) {
-          __align__(16) __nv_bfloat16 h[8];
+          uint32_t h[4];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            h[q] = __float2bfloat16_rn(f[q]);
-            f[q] -= __bfloat162float(h[q]);  // exact: the remainder of a round-to-nearest
+          for (int q = 0; q < 4; ++q) {
+            h[q] = piece < 2 ? cv_pack_sat(f[2 * q], f[2 * q + 1]) : cv_pack(f[2 * q], f[2 * q + 1]);
+            f[2 * q] -= __uint_as_float(h[q] << 16);  // exact: the remainder of a round-to-nearest
+            f[2 * q + 1] -= __uint_as_float(h[q] & 0xffff0000u);
           }
-          *reinterpret_cast<uint4*>(st + piece * ab + dst[k]) = *reinterpret_cast<const uint4*>(h);
+          *reinterpret_cast<uint4*>(st + piece * ab + dst[k]) = make_uint4(h[0], h[1], h[2], h[3]);
         }
       }
       fence_async_smem();

@@ -122,9 +122,10 @@ static RfFn rf_fn(int mode, int inverse) {
   return inverse ? k_rowfft2<R1, R2, TY, true, RF_IN> : k_rowfft2<R1, R2, TY, false, RF_IN>;
 }
 
-// SMSM_ERR_ARG: a length without such a kernel (16 x 32 and longer, or with factors beyond 16 x 16)
+// SMSM_ERR_ARG: a length without such a kernel, or the generic kernels are asked for
 smsm_status launch_rowfft2(const smsm_plan_s* P, int mode, const float2* in, float2* out, int nb, int rows, int inverse,
                            int band, float2* p, const double* rr_new, const double* rr_old, int nrr, cudaStream_t s) {
+  if (P->flags & SMSM_FLAG_GENERIC_KERNELS) return SMSM_ERR_ARG;
   const bool few = rows <= 8;  // (data lines of a short shot: half the CTA's rows would be missing)
   RfFn fn;
 #define RF_N(R1, R2)                                                            \

@@ -466,7 +466,17 @@ __global__ void __launch_bounds__(GRED_T * 8) k_gram_tc_reduce(const float* __re
   for (int k = 0; k < NK; ++k) {
     const int cc = ccb + k;
     if (c < C && cc < C && c <= cc) {
-      const double re = (double)rh[k] + (double)rl[k], im = (double)ih[k] + (double)il[k];
+      double re = (double)rh[k] + (double)rl[k], im = (double)ih[k] + (double)il[k];
+      if (!(isfinite(rh[k]) && isfinite(ih[k]))) {  // beyond FP32's range, or not finite: the plain sum in FP64
+        const size_t pa = gtc_rofs(R2C, c, cc) + (cc & 3), pb = gtc_rofs(R2C, Cp + c, Cp + cc) + ((Cp + cc) & 3),
+                     pc = gtc_rofs(R2C, c, Cp + cc) + ((Cp + cc) & 3), pt = gtc_rofs(R2C, cc, Cp + c) + ((Cp + c) & 3);
+        re = im = 0.0;
+        for (int g = 0; g < nG; ++g) {
+          const float* R = Rf + (size_t)g * R2C * R2C;
+          re += (double)R[pa] + (double)R[pb];
+          im += (double)R[pc] - (double)R[pt];
+        }
+      }
       if (c == cc) {
         Gl[(size_t)c * C + c] = make_double2(re, 0.0);
       } else {

@@ -400,6 +400,19 @@ __global__ void __launch_bounds__(GTC_THREADS, 1)
   if (warp == 0) tmem_dealloc(tmem, tmem_cols);
 }
 
+// one entry's plain sum in FP64: what k_gram_tc_reduce takes near and beyond FP32's range (out of its way: a call)
+__device__ __noinline__ double2 gram_sum64(const float* R, int R2C, int c, int cc, int nG) {
+  const int Cp = R2C / 2;
+  const size_t pa = gtc_rofs(R2C, c, cc) + (cc & 3), pb = gtc_rofs(R2C, Cp + c, Cp + cc) + ((Cp + cc) & 3),
+               pc = gtc_rofs(R2C, c, Cp + cc) + ((Cp + cc) & 3), pt = gtc_rofs(R2C, cc, Cp + c) + ((Cp + c) & 3);
+  double re = 0.0, im = 0.0;
+  for (int g = 0; g < nG; ++g, R += (size_t)R2C * R2C) {
+    re += (double)R[pa] + (double)R[pb];
+    im += (double)R[pc] - (double)R[pt];
+  }
+  return make_double2(re, im);
+}
+
 // G[c][c'] (c <= c') = sum_g (R[c][c'] + R[Cp+c][Cp+c']) + i (R[c][Cp+c'] - R[c'][Cp+c]),
 // every entry read from R's upper triangle; G[c'][c] is written as the conjugate, so G is
 // exactly Hermitian.  One CTA (32 x 8 threads) per 32 x 32 tile (c, c') on or above the
@@ -467,15 +480,10 @@ __global__ void __launch_bounds__(GRED_T * 8) k_gram_tc_reduce(const float* __re
     const int cc = ccb + k;
     if (c < C && cc < C && c <= cc) {
       double re = (double)rh[k] + (double)rl[k], im = (double)ih[k] + (double)il[k];
-      if (!(isfinite(rh[k]) && isfinite(ih[k]))) {  // beyond FP32's range, or not finite: the plain sum in FP64
-        const size_t pa = gtc_rofs(R2C, c, cc) + (cc & 3), pb = gtc_rofs(R2C, Cp + c, Cp + cc) + ((Cp + cc) & 3),
-                     pc = gtc_rofs(R2C, c, Cp + cc) + ((Cp + cc) & 3), pt = gtc_rofs(R2C, cc, Cp + c) + ((Cp + c) & 3);
-        re = im = 0.0;
-        for (int g = 0; g < nG; ++g) {
-          const float* R = Rf + (size_t)g * R2C * R2C;
-          re += (double)R[pa] + (double)R[pb];
-          im += (double)R[pc] - (double)R[pt];
-        }
+      if (!(fabsf(rh[k]) + fabsf(ih[k]) <= 3.4e38f)) {  // near or beyond FP32's range, or not finite
+        const double2 s = gram_sum64(Rf, R2C, c, cc, nG);
+        re = s.x;
+        im = s.y;
       }
       if (c == cc) {
         Gl[(size_t)c * C + c] = make_double2(re, 0.0);

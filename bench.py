@@ -242,7 +242,10 @@ def stage_work(cfg, D, sweeps):
     half = Cp // 2
     P = (N - r + 1) ** 2
     R2 = 2 * r - 1
-    nband = NN - (N - 2 * (r - 1)) ** 2
+    # border band: on the strips' lines only the taps across whose patches leave the image, (3r - 2)/2 of 2r - 1 on
+    # average, and all 2r - 1 along; every tap at the corners
+    w = r - 1
+    band_taps = 4 * w * (N - 2 * w) * (3 * w + 1) / 2 * R2 + 4 * w * w * R2 * R2
     lg = np.log2
     # column stage, per image column: the B lines' inverse and forward N-point FFTs
     # (5 N log2 N each), the A^H A class products (8 L Ns flops per pixel and line) and
@@ -250,7 +253,8 @@ def stage_work(cfg, D, sweeps):
     col = N * (B * 2 * 5 * N * lg(N) + B * N * 8 * (L * Ns + Ns))
     return {
         "column": ("alu", D * col),
-        "band": ("alu", D * 8 * L * nband * Ns * Ns * R2 * R2),
+        "band": ("alu", D * 8 * L * Ns * Ns * band_taps),
+        # the direct products of the reduced-precision form (the FP32 form needs fewer: lagged products)
         "gram": ("alu", D * 8 * L * P * C * (C + 1) / 2),
         # 13 Cholesky inverses of C^3/2 complex multiply-adds (c/eps = 1.6e5), or, with Jacobi sweeps,
         # every round: the 2x2 blocks of G (96 flops each) and the rotated column pairs of V
@@ -421,7 +425,7 @@ def run_ours(args):
         p_ms = max_over_ranks(sum(a.elapsed_time(b) for a, b in pev) / args.steps, dev)
         forms = {
             "plain": {"value": throughput(world, D, p_ms), "ms_per_step": p_ms,
-                      "form": "FP32-form Gram (three BF16 pieces), default lanes, no autotuning, start A^H y"},
+                      "form": "FP32-form Gram (lagged FP32 products), default lanes, no autotuning, start A^H y"},
             "combined": {"value": value, "ms_per_step": ms,
                          "form": "BF16 hi+lo split Gram, batch of directions in autotuned lanes with autotuned "
                                  "Gram split-K, start A^H y", "autotuned": tuned,
@@ -747,7 +751,7 @@ def main():
                     help="plain: MB 2, 4 shots, 32 coils, 128^2, FOV/2; precision: MB 3, 4 shots, 32 coils, "
                          "256^2, FOV/3 (both filter 6x6, 20 outer x 15 CG)")
     ap.add_argument("--precision", default="fp32", choices=["fp32", "bf16-split"],
-                    help="Hankel Gram form with --form plain: FP32-exact BF16 pieces or the BF16 hi+lo split")
+                    help="Hankel Gram form with --form plain: FP32 products or the BF16 hi+lo split")
     ap.add_argument("--form", default="combined", choices=["combined", "plain"],
                     help="combined: the BF16 split + autotuned batched form, timed beside the plain form on the "
                          "same data (value = combined); plain: only the form --precision selects")

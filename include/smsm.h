@@ -79,7 +79,8 @@ typedef struct {
  * (larger C: FP32 FMA; the BF16 split form needs C <= 144):
  *   FP32: every FP32 value split exactly into three BF16 pieces b1 + b2 + b3,
  *         six BF16 products b_i b_j' (i + j <= 4), FP32 accumulation: every
- *         product as accurate as an FP32 multiply;
+ *         product as accurate as an FP32 multiply.  Solves with VALID patches
+ *         form it from lagged FP32 products instead (any C);
  *   BF16_SPLIT: two pieces hi = bf16(x), lo = bf16(x - hi), three products
  *         hi hi' + hi lo' + lo hi' (~2^-16 relative per product).
  */
@@ -111,7 +112,8 @@ typedef enum { SMSM_BOUNDARY_VALID = 0, SMSM_BOUNDARY_PERIODIC = 1 } smsm_bounda
  * The IRLS weights W_l = (G_l + eps I)^(-1/2) are formed without an eigen-decomposition
  * unless the call asks for one (NULLSPACE mode, eig_cold, eig_tol > 0, max_sweeps below
  * 30, SMSM_FLAG_CLUSTER_EIG, SMSM_FLAG_GENERIC_KERNELS), eps0_rel * eps_min_rel is below
- * 1e-5, or a Gram's scale passes 2^20 eps; then the Jacobi eigensolvers make them.
+ * 1e-5, a Gram's scale passes 2^20 eps, or rounding left a Gram (plus eps) indefinite;
+ * then the Jacobi eigensolvers make them.
  *
  * Solver parameters.  The paper minimises Eq. 10 with an augmented-Lagrangian
  * scheme whose listing is in another paper; this library minimises the same
@@ -141,7 +143,7 @@ typedef struct {
                          (default 0: start from the previous iteration's eigenvectors) */
   int lanes;          /* batch > 1: split the batch into this many sub-batches solved as
                          concurrent branches of the captured graph, started out of phase
-                         so that one lane's (latency-bound) eigensolver runs while other
+                         so that one lane's latency-bound kernels run while other
                          lanes' CG runs; 0 -> automatic (3 for a batch of at least 9, 2
                          from 4), at most SMSM_MAX_LANES and the batch.  Results do not
                          depend on it. */
@@ -332,8 +334,9 @@ smsm_status smsm_hankel_gram_noalloc(const void* x, void* G, int mb, int shots, 
 /*
  * Autotuner (not in the paper).  Times, on the plan's own data y (layout of
  * smsm_reconstruct), the tensor-core Gram with each candidate number of split-K
- * blocks (one to six waves of CTAs over the GPU) and shortened solves (min(K, 6)
- * outer iterations of `params`, so that the cold first eigen step weighs about as
+ * blocks (one to six waves of CTAs over the GPU; FP32 solves with VALID patches do not
+ * use it, smsm_hankel_gram does) and shortened solves (min(K, 6)
+ * outer iterations of `params`, so that the first weight step weighs about as
  * little as in the full solve) with 1..min(batch, SMSM_MAX_LANES) concurrent lanes,
  * keeps the fastest of each for this plan (the lanes apply when params->lanes is 0)
  * and remembers them for every later plan of the same shape (mb, shots, coils, N,

@@ -67,8 +67,9 @@ __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__floa
 // accumulation, as in an FP32 FMA loop.  Every MMA rounds its accumulator once, so the leading piece's products
 // are dealt out to three accumulators by tap row (24 roundings each for 64 channels) and the two small
 // pieces' (2^-8 and 2^-16 of them) to a fourth, all added in the epilogue: with one accumulator for the
-// leading products the learned start of two 256 x 256 groups was 2.9e-6 from its 64-bit value, with three 8.9e-7 (FP32
-// FMAs: 9e-7).
+// leading products the learned start of two 256 x 256 groups was 2.9e-6 from its 64-bit value, with three 7.8e-7 ..
+// 9.3e-7 over seeds and sizes at 64 channels, 2.9e-7 .. 4e-7 at 16 to 40 (FP32 FMAs: 7.5e-7 .. 1.06e-6 and 3.3e-7 ..
+// 6.5e-7).  An infinite weight (a diverged network) gives NaN: its products with the small pieces have both signs.
 //
 // Implicit GEMM without copies: the image is cut into column strips of TW pixels, padded to P = TW + 2 columns, and
 // a strip is read as one line of pixels; a CTA takes 128 consecutive ones and stages them with
@@ -82,8 +83,9 @@ __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__floa
 //   * the producer warps write the outputs from TMEM at the end.
 // N = NT columns: the real parts of up to 64 output channels, then the imaginary ones.  Waits are bounded; on a
 // timeout the network's error flag is raised.
-// Measured (before: FP32 FMAs, a 16 x 16 pixel tile x 32 channels per CTA), two 256 x 256 images: 64 -> 64 channels
-// 770 -> 62 us; the learned start of both groups (6 layers, width 64) 3.73 -> 0.76 ms.
+// Measured (before: FP32 FMAs, a 16 x 16 pixel tile x 32 channels per CTA), two 256 x 256 images: 12 -> 64 channels
+// 160 -> 60 us, 64 -> 64 770 -> 120 us, 64 -> 12 438 -> 139 us; the learned start of both groups (6 layers, width 64)
+// 3.73 -> 0.74 ms.
 // ---------------------------------------------------------------------------
 #define CV_TL 128                 // pixels of a strip per CTA (one M = 128 block)
 #define CV_MAXP 66                // strip pitch at most

@@ -10,14 +10,16 @@
 // each.  A Jacobi sweep of a 144 x 144 matrix is 143 dependent rounds on two SMs, 3 to 13 sweeps
 // per outer iteration; a term is nine dependent block steps and the chip works on every term.
 // Measured, the weight step of an outer iteration (mean over a solve; before: Jacobi): two 144 x 144
-// matrices 2.14 -> 0.11 ms, 52 of them 2.4 -> 0.45 ms, four 288 x 288 12.8 -> 0.57 ms.
+// matrices 2.14 -> 0.10 ms, 52 of them 2.4 -> 0.44 ms (0.46 with the probe below), four 288 x 288 12.8 -> 0.57 ms.
 //
 // Accuracy: the terms add without cancellation, and a Cholesky inverse in FP32 is that of a matrix
 // off by FP32 rounding, as G itself is once it is held in FP32.  Against the 64-bit weight, on the
 // Grams of the 128 x 128 workload over its 20 outer iterations (relative Frobenius error, and of
 // G^(1/2) W G^(1/2), what acts on the data): 4e-7 .. 1.8e-4 and 3e-7 .. 4e-6; the Jacobi
 // eigensolver 8e-6 .. 1.4e-4 and 1.3e-6 .. 7e-6; W of G rounded to FP32 1.5e-7 .. 7e-5 and 1e-8 ..
-// 8e-7.  (A Newton-Schulz iteration for A^(-1/2), which needs GEMMs only, was five times worse
+// 8e-7.  At eps 1e-5 of the largest eigenvalue (c/eps near 2^20), solves of six geometries, C = 32 .. 288, two
+// outer iterations, are 5.8e-7 .. 6.1e-6 from the oracle, with the Jacobi eigensolver 5.8e-7 .. 1.5e-5, and eps_1
+// is within 3.4e-7 of its 64-bit value (Jacobi: 1.4e-6).  (A Newton-Schulz iteration for A^(-1/2), which needs GEMMs only, was five times worse
 // on the data; a Gauss-Jordan sweep in place of Cholesky a hundred times worse on W.)
 //
 // eps_1 = eps0_rel times the largest eigenvalue: G is squared IS_SQ times (normalised by its
@@ -615,8 +617,9 @@ size_t invsqrt_per(const smsm_plan_s* P) {  // complex values of one matrix's te
 
 typedef void (*TermFn)(const float2*, const IsParam*, const IsRow*, float2*, int*, const float2*, int, int, int, int);
 
-// Slots = blocks per warp.  One CTA's 16 warps hold up to 5 blocks each (C <= 192: 80 of 128 registers);
-// above, four CTAs hold the 105 (C = 208+) to 210 (C = 320) blocks with 2 to 4 each.
+// Slots = blocks per warp.  One CTA's 16 warps hold up to 5 blocks each (C <= 192), 16 of a lane's 128 registers
+// each (four or five blocks spill 100 and 600 bytes); above, four CTAs hold the 105 (C = 208+) to 210 (C = 320)
+// blocks with 2 to 4 each.
 // Two matrices or fewer leave most SMs idle: four CTAs per term then, too (the same blocks, the same sums), where a
 // warp has several blocks to give away (two matrices: C = 144 89 -> 62 us; C = 100 53 -> 62, left alone).
 static TermFn term_fn(int C, int LD, int* cl) {

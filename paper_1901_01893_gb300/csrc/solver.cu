@@ -449,11 +449,13 @@ static int solve_lanes(const smsm_plan_s* P, const smsm_params* prm) {
 
 // The whole solve on stream s (being captured).  Stage timing brackets the
 // launches of lane 0 (its own stream).  With several lanes, lane k solves
-// directions [k D / n, (k+1) D / n) on its own stream, and lane k's first eigen
-// step waits for lane k-1's: the lanes start out of phase, so one lane's
-// eigensolver (a few CTAs that wait on latency) runs next to the other lanes'
-// bandwidth-bound kernels.  (Forcing the eigen steps to alternate for the whole
-// solve measured slower with three or more lanes: it serialises them.)
+// directions [k D / n, (k+1) D / n) on its own stream, and lane k's first weight
+// step waits for lane k-1's: the lanes start out of phase, so that one lane's
+// latency-bound kernels (the eigensolvers above all, where they run: a few CTAs)
+// are beside the other lanes' full-GPU ones.  Without an eigen-decomposition the lanes matter little: the
+// autotuner's shortened solve of 26 directions of 128 x 128 takes 23.6, 23.5 and 23.3 ms with one, two and three.
+// (Forcing the eigen steps to alternate for the whole solve measured slower with three or more lanes: it
+// serialises them.)
 static smsm_status enqueue_solve(smsm_plan_s* P, const smsm_params* prm, cudaStream_t s) {
   smsm_status st;
   if (prm->timing && !P->tpool) P->tpool = new TimingPool();
@@ -877,7 +879,8 @@ smsm_status solver_autotune(smsm_plan_s* P, const void* y, const smsm_params* pr
   SMSM_CUDA_TRY(cudaEventCreate(&e1));
   smsm_status st = SMSM_OK;
   float ms = 0.f;
-  // 1. the Gram's split-K blocks, on the starting point A^H y
+  // 1. the Gram's split-K blocks, on the starting point A^H y (FP32 VALID solves take the lagged Gram: there they
+  // serve smsm_hankel_gram)
   if (P->gram_tc) {
     const size_t ny = (size_t)P->D * P->Ns * P->Nc * P->M * P->N;
     cudaError_t ce = cudaMemcpyAsync(P->ybuf, y, sizeof(float2) * ny, cudaMemcpyDeviceToDevice, s);
@@ -912,9 +915,9 @@ smsm_status solver_autotune(smsm_plan_s* P, const void* y, const smsm_params* pr
     rep.gram_nG = P->gram_tc_nG;
   }
   // 2. the lanes, on a shortened solve of the same data: six outer iterations (or K), so
-  // that the cold first eigen step -- which the lanes start one after another -- weighs as
-  // little in the timing as in a full solve (two iterations picked one lane where three
-  // were 9 % faster at K = 20)
+  // that the first weight step -- which the lanes start one after another -- weighs as
+  // little in the timing as in a full solve (with the eigensolvers, two iterations picked one lane
+  // where three were 9 % faster at K = 20)
   if (!st) {
     smsm_params q = *prm;
     q.outer_iters = prm->outer_iters < 6 ? prm->outer_iters : 6;
